@@ -495,9 +495,11 @@ dg_status degrid_execute_noalloc(void *stream, int nx, int ny, int nz,
  * subgrid_predict_plan_create
  *   n                  image and subgrid side N: even, >= 8, N * N * nz < 2^31
  *   nz                 w-planes per subgrid, 1 .. 64 (4 for the paper's stack)
- *   subgrids_per_pass  subgrids transformed together (1 .. 4096); the plan
- *                      holds a work buffer of subgrids_per_pass * nz * N * N
- *                      complex64 and a batched 2D FFT plan (cuFFT)
+ *   subgrids_per_pass  subgrids transformed together at most (1 .. 4096);
+ *                      the plan holds a work buffer of no more than that many
+ *                      (nz * N * N complex64 each) and, for sizes without a
+ *                      transform of the library's own, a batched 2D FFT plan
+ *                      (cuFFT)
  *   device             CUDA device ordinal
  * Returns DG_OK, DG_ERR_ARG, DG_ERR_OOM or DG_ERR_CUDA.
  *

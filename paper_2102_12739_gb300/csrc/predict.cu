@@ -14,7 +14,9 @@
 // at nz consecutive w-planes, stored [y][x][c] like the stack the degridding
 // kernels read.
 //
-// Per pass of up to P subgrids, three steps on the caller's stream:
+// Sizes and plane counts that predict_fft.cu covers take its two kernels
+// (screen and row transforms, column transforms and window).  The others
+// take, per pass of up to P subgrids, three steps on the caller's stream:
 //  1. screen_kernel (hand-written): for every pixel and subgrid, the tapered
 //     image times the w-phase screen of each plane and (-1)^(a + b) into a
 //     work buffer [P][nz][N][N].  The phase w (n - 1) runs to hundreds of
@@ -40,17 +42,23 @@
 #include <new>
 
 #include "internal.cuh"
+#include "predict_fft.cuh"
+#include "predict_fft.h"
 
 struct subgrid_predict_plan {
     int device;
     int n, nz, per_pass;
     cufftHandle fft;
     bool fft_ok;
+    dg_predict_fft *fused;      // the fused transform, where there is one for n and nz (the rest is unused then)
     float2 *work;       // [per_pass][nz][n][n]
     float2 *nm1;        // [n][n]: n - 1 per pixel as (hi, lo) floats, hi NaN outside the unit circle
 };
 
 namespace {
+
+using dg::cmul;
+using dg::screen_phasor;
 
 constexpr int kThreads = 256;
 
@@ -71,25 +79,6 @@ __global__ void nm1_kernel(float2 *__restrict__ nm1, int n, double dl)
     } else {
         nm1[i] = make_float2(__int_as_float(0x7fc00000), 0.f);
     }
-}
-
-// exp(-2 pi i w (n - 1)) with w = (w_hi + w_lo) and n - 1 = (n_hi + n_lo):
-// the turns of the product are reduced to [-1/2, 1/2] in double-float
-// arithmetic (|w (n - 1)| < 2^22 turns), then rotated in FP32.
-__device__ __forceinline__ float2 screen_phasor(float w_hi, float w_lo, float2 nm)
-{
-    const float p = w_hi * nm.x;
-    const float e = fmaf(w_hi, nm.x, -p);                   // p + e = w_hi * n_hi exactly
-    const float c = fmaf(w_hi, nm.y, w_lo * nm.x);          // cross terms (w_lo * n_lo dropped)
-    const float f = (p - rintf(p)) + (e + c);               // p - rint(p) is exact
-    float s, co;
-    sincospif(2.0f * f, &s, &co);
-    return make_float2(co, -s);
-}
-
-__device__ __forceinline__ float2 cmul(float2 a, float2 b)
-{
-    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 
 // Step 1: grid (ceil(N / kThreads), N rows); thread (a, b) makes pixel (a, b)
@@ -209,6 +198,7 @@ struct DeviceGuard {
 
 void free_plan(subgrid_predict_plan *p)
 {
+    dg_predict_fft_destroy(p->fused);
     if (p->fft_ok)
         cufftDestroy(p->fft);
     cudaFree(p->work);
@@ -245,6 +235,16 @@ dg_status subgrid_predict_plan_create(subgrid_predict_plan_t *out, int n, int nz
     p->fft_ok = false;
     p->work = nullptr;
     p->nm1 = nullptr;
+    p->fused = nullptr;
+    if (dg_predict_fft_supported(n, nz)) {
+        const cudaError_t err = dg_predict_fft_create(&p->fused, n, nz, subgrids_per_pass, device);
+        if (err != cudaSuccess) {
+            delete p;
+            return from_cuda(err);
+        }
+        *out = p;
+        return DG_OK;
+    }
     const size_t np = (size_t)n * n;
     cudaError_t e = cudaMalloc((void **)&p->work, sizeof(float2) * np * nz * subgrids_per_pass);
     if (e == cudaSuccess)
@@ -296,7 +296,9 @@ dg_status subgrid_predict_execute(subgrid_predict_plan_t p, void *stream, double
     if (!guard.ok)
         return DG_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
-    const int64_t np = (int64_t)p->n * p->n;
+    if (p->fused)
+        return from_cuda(dg_predict_fft_execute(p->fused, st, theta, image, taper, n_subgrids, uv_offsets, w_planes,
+                                                subgrids_out));
     nm1_kernel<<<dim3((unsigned)((p->n + kThreads - 1) / kThreads), (unsigned)p->n), kThreads, 0, st>>>(
         p->nm1, p->n, theta / p->n);
     cudaError_t e = cudaGetLastError();

@@ -61,6 +61,26 @@ def test_small_stacks_every_cell(n, nz, theta, per_pass):
         assert rel_l2(got[s], ref[s]) <= TOL, (s, rel_l2(got[s], ref[s]))
 
 
+@pytest.mark.parametrize("n,nz,S,per_pass", [
+    (64, 4, 5, 4), (96, 8, 3, 2), (128, 4, 3, 2), (192, 12, 2, 1), (256, 4, 3, 8), (320, 4, 2, 1), (384, 8, 2, 2),
+    (400, 4, 3, 2), (512, 4, 3, 1), (768, 4, 2, 2), (1024, 4, 1, 1),
+    (72, 4, 2, 2), (64, 6, 2, 2),               # no fused transform: the library's
+])
+def test_every_transform_size(n, nz, S, per_pass):
+    # each size of the fused transform: one and several plane groups, a ragged
+    # last pass, windows that wrap on both axes, a plane spacing that changes
+    # between items, pixels outside the unit circle (theta 1.6)
+    rng = np.random.default_rng(n + nz)
+    img = (rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))).astype(np.complex64)
+    taper = rng.uniform(0.5, 2.0, (n, n)).astype(np.float32) if nz != 8 else None
+    uv = np.array([[1, -n // 2], [-3 * n + 5, n - 1], [0, 0], [n // 2, 7], [-1, -1]], dtype=np.int32)[:S]
+    w = np.array([[812.5, 3.0], [-40000.0, 3.0], [11.0, -250.75], [0.0, 0.0], [5.0, 1.0]])[:S]
+    got = run(img, 1.6, uv, w, nz, taper, per_pass)
+    ref = P.predict(img, 1.6, np.concatenate([uv, w], axis=1), nz=nz, taper=taper)
+    for s in range(S):
+        assert rel_l2(got[s], ref[s]) <= TOL, (s, rel_l2(got[s], ref[s]))
+
+
 def test_passes_of_more_than_256_subgrids():
     # a pass of 300 subgrids: the screen kernel splits the subgrids' w in
     # tiles of 256; plane spacings equal within runs and changing between
