@@ -10,7 +10,7 @@
 #include "internal.cuh"
 
 cudaError_t dg_launch_pack(cudaStream_t st, dg_dtype dtype, int n_subgrids, int64_t elems,
-                           const float *in, void *codes_out, float *scale_out, int sm_count);
+                           const float *in, void *codes_out, float *scale_out);
 
 namespace {
 
@@ -669,12 +669,8 @@ dg_status degrid_pack_subgrids(void *stream, dg_dtype dtype, int n_subgrids, int
         return DG_ERR_ARG;
     if (n_subgrids == 0)
         return DG_OK;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return DG_ERR_CUDA;
     return from_cuda(dg_launch_pack((cudaStream_t)stream, dtype, n_subgrids, elems, in, codes_out,
-                                    scale_out, sms));
+                                    scale_out));
 }
 
 dg_status degrid_get_status(degrid_plan_t p, void *stream, int64_t *n_invalid)

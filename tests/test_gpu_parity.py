@@ -1073,3 +1073,38 @@ def test_sparse_and_dense_lists_at_every_chunk_size():
     assert rel_l2(outs[0][idx], ref) <= TOL["c64"]
     gref, _ = oracle.grid(G_UV, G_W, synth.SUBGRID_SHAPE, len(counts), w.uvw, w.vis_offsets, yv)
     assert rel_l2(g, gref) <= TOL["c64"]
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("S,elems,shift", [
+    (1, 1, 0), (3, 3, 0), (2, 8192, 0), (2, 8193, 0), (2, 8192, 1),     # one and two pieces; no 16-byte loads
+    (70, 60000, 0), (9, 512 * 512 * 4, 0),                              # several groups of subgrids
+])
+def test_packing_every_form_bitwise(dtype, S, elems, shift):
+    # codes and scales against torch's correctly rounded division and
+    # conversions; an all-zero subgrid, infinities and a subnormal maximum
+    d = dev()
+    g = torch.Generator(device=d)
+    g.manual_seed(S * 31 + elems)
+    flat = torch.randn(S * elems + shift, 2, generator=g, device=d)
+    x = torch.view_as_complex(flat)[shift:].view(S, elems, 1, 1)       # shift 1: 8 bytes off a 16-byte boundary
+    if S == 9:
+        # exponents over the whole range: quotients down to and below the
+        # smallest normal number, and halfway cases of the 16-bit formats
+        e = torch.randint(-149, 3, x.shape, generator=g, device=d).float()
+        torch.view_as_real(x)[3:6] = torch.ldexp(torch.view_as_real(x)[3:6], e[3:6, ..., None])
+        torch.view_as_real(x)[6] = (torch.view_as_real(x)[6] * 2048).round() / 2048
+        torch.view_as_real(x)[7, :, 0, 0, 0] = -0.0
+    if S > 1:
+        torch.view_as_real(x)[1] = 0.0
+    if S > 2:
+        torch.view_as_real(x)[2] *= 1e-40
+        torch.view_as_real(x)[0, 0, 0, 0, 1] = float("inf")
+    codes, scale = dg.pack_subgrids(x, dtype)
+    r = torch.view_as_real(x)
+    want = r.abs().amax(dim=(1, 2, 3, 4))
+    assert torch.equal(scale, want)
+    q = torch.where(want[:, None, None, None, None] > 0, r / want[:, None, None, None, None], torch.zeros_like(r))
+    q = q.to(codes.dtype)
+    same = (codes == q) | (codes.isnan() & q.isnan())
+    assert bool(same.all())
