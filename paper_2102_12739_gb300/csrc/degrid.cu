@@ -39,6 +39,7 @@
 // The products use packed FFMA2 on (re, im) pairs with a duplicated real
 // weight: bitwise the same as two scalar FMAs, in half the instructions
 // (11.2 instead of 12.7 warp instructions per visibility on dense lines).
+#include "footprint.cuh"
 #include "pipeline.cuh"
 
 namespace dg {
@@ -61,35 +62,6 @@ struct alignas(128) WarpSmem {
 // M[2j + i][a] for i = 0, 1 and a = 0..7 of footprint `key` (subgrid at
 // `base`) with w row gw: lane (a = lane & 7, b = lane >> 3 and b + 4)
 // computes two entries into shared memory, then every lane reads its rows.
-// sum_c g_w[c] s[e + c] for one footprint point (the entries of M; the
-// direct arm forms them the same way, so both arms round alike).
-// With `vec` (16-byte aligned subgrids, nz a multiple of the elements per
-// 16 bytes, and a footprint start z0 that is one too) the four elements are
-// read with 16-byte loads.
-template <int DT>
-__device__ __forceinline__ float2 footprint_point(const void *sub, int64_t e, const float4 &gw, bool vec)
-{
-    float2 s[4];
-    if (vec) {
-        Storage<DT>::load4(sub, e, s);
-    } else {
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-            s[c] = Storage<DT>::load(sub, e + c);
-    }
-    float2 m;
-    m.x = fmaf(s[3].x, gw.w, fmaf(s[2].x, gw.z, fmaf(s[1].x, gw.y, s[0].x * gw.x)));
-    m.y = fmaf(s[3].y, gw.w, fmaf(s[2].y, gw.z, fmaf(s[1].y, gw.y, s[0].y * gw.x)));
-    return m;
-}
-
-// Whether the footprint starting at `key` can use 16-byte loads.
-template <int DT>
-__device__ __forceinline__ bool vec_footprint(bool vec_ok, int key)
-{
-    return vec_ok && (key % Storage<DT>::kQuad) == 0;
-}
-
 template <int DT>
 __device__ __forceinline__ void build_rows(float2 (&M)[2][8], float2 (&mbuf)[8][8], const void *sub,
                                            int64_t base, int key, const float4 &gw, const Geometry &g,
@@ -133,34 +105,6 @@ __device__ __forceinline__ float2 quarter_sum(const float2 (&M)[2][8], const Row
     return __ffma2_rn(t1, make_float2(v.y, v.y), __fmul2_rn(t0, make_float2(v.x, v.x)));
 }
 
-// 2D G_uv table: this lane's quarter sum_{i} sum_a G[blk][2j + i][a] M[i][a]
-// with the 16 weights of rows 2j, 2j + 1 of the visibility's block read
-// straight from the (L2-resident) table.
-__device__ __forceinline__ float2 quarter_sum_2d(const float2 (&M)[2][8], const float *__restrict__ g2,
-                                                 int blk, int j)
-{
-    const float4 *w = reinterpret_cast<const float4 *>(g2 + (size_t)blk * (kUV * kUV) + 2 * kUV * j);
-    const float4 w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2), w3 = __ldg(w + 3);
-    const float g0[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-    const float g1[8] = {w2.x, w2.y, w2.z, w2.w, w3.x, w3.y, w3.z, w3.w};
-    float2 t0 = __fmul2_rn(M[0][0], make_float2(g0[0], g0[0]));
-    float2 t1 = __fmul2_rn(M[1][0], make_float2(g1[0], g1[0]));
-#pragma unroll
-    for (int a = 1; a < 8; ++a) {
-        t0 = __ffma2_rn(M[0][a], make_float2(g0[a], g0[a]), t0);
-        t1 = __ffma2_rn(M[1][a], make_float2(g1[a], g1[a]), t1);
-    }
-    return __fadd2_rn(t0, t1);
-}
-
-// One pass: the separable sum from the staged rows, or the 2D table sum.
-template <bool T2D>
-__device__ __forceinline__ float2 pass_sum(const float2 (&M)[2][8], const RowStage &S,
-                                           const float *__restrict__ g2, int r, int blk, int j)
-{
-    return T2D ? quarter_sum_2d(M, g2, blk, j) : quarter_sum(M, S, r, j);
-}
-
 // Direct arm: this lane's quarter of visibility r (footprint `key`, w row gw)
 // from the subgrid itself, M's two rows formed on the fly; the same
 // operations in the same order as build_rows followed by quarter_sum.
@@ -189,15 +133,6 @@ __device__ __forceinline__ float2 quarter_sum_direct(const void *sub, int64_t ba
         t1 = __ffma2_rn(m1[a], make_float2(gu[a], gu[a]), t1);
     }
     return __ffma2_rn(t1, make_float2(v.y, v.y), __fmul2_rn(t0, make_float2(v.x, v.x)));
-}
-
-// Error-free sum (Knuth's TwoSum): a + b = s + e exactly, s = fl(a + b).
-__device__ __forceinline__ float two_sum(float a, float b, float &e)
-{
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    return s;
 }
 
 // State of the cached footprint matrix: rows 2j, 2j + 1 of M for (key, fw)
@@ -247,13 +182,12 @@ __device__ __forceinline__ void reduce_store(float2 (&P)[4], const Batch &h, flo
 }
 
 
-template <int DT, bool COMP, bool DIRECT, bool T2D>
+template <int DT, bool COMP, bool DIRECT>
 __device__ __forceinline__ void sum_half(MState &ms, WarpSmem &ws, const RowStage &S, const Issued &I,
                                          const Batch &h, const void *__restrict__ subgrids, int64_t base,
                                          float sc, const Geometry &g, const float4 *wtab,
                                          const float *__restrict__ gwt, float2 *__restrict__ vis_out,
-                                         int direct_runs, bool vec_ok, const float *__restrict__ g2,
-                                         int lane, int p, int j)
+                                         int direct_runs, bool vec_ok, int lane, int p, int j)
 {
     float2 P[4];                        // pass k: this lane's quarter of visibility 8 (k ^ j) + p
     if (I.uniform) {
@@ -266,9 +200,9 @@ __device__ __forceinline__ void sum_half(MState &ms, WarpSmem &ws, const RowStag
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int r = 8 * (k ^ j) + p;
-            P[k] = pass_sum<T2D>(ms.M, S, g2, r, T2D ? __shfl_sync(kFull, I.blk, r) : 0, j);
+            P[k] = quarter_sum(ms.M, S, r, j);
         }
-    } else if (DIRECT && !T2D && I.runs >= direct_runs) {
+    } else if (DIRECT && I.runs >= direct_runs) {
         // Short runs: every visibility is summed from its own footprint
         // (pass k covers visibilities 8k .. 8k + 7; invalid ones stay zero).
         // Pays off when the footprints of a half overlap (slowly moving
@@ -322,7 +256,7 @@ __device__ __forceinline__ void sum_half(MState &ms, WarpSmem &ws, const RowStag
                     ms.key = lk;
                     ms.fw = lf;
                 }
-                const float2 x = pass_sum<T2D>(ms.M, S, g2, r, T2D ? __shfl_sync(kFull, I.blk, r) : 0, j);
+                const float2 x = quarter_sum(ms.M, S, r, j);
                 const bool mine = !done && kr == lk && fr == lf;
                 if (mine)
                     acc = x;
@@ -342,14 +276,14 @@ __device__ __forceinline__ void sum_half(MState &ms, WarpSmem &ws, const RowStag
 // Both halves of a full step share one footprint and w row (the common
 // case on dense lists): their eight passes are summed in one block, so the
 // scheduler can interleave the two halves' loads and FMA chains.
-template <int DT, bool COMP, bool T2D>
+template <int DT, bool COMP>
 __device__ __forceinline__ void sum_step_uniform(MState &ms, WarpSmem &ws, const RowStage &S0,
                                                  const RowStage &S1, const Issued &I0, const Issued &I1,
                                                  const Batch &b, const void *__restrict__ subgrids,
                                                  int64_t base, float sc, const Geometry &g,
                                                  const float4 *wtab, const float *__restrict__ gwt,
                                                  float2 *__restrict__ vis_out, bool vec_ok,
-                                                 const float *__restrict__ g2, int lane, int p, int j)
+                                                 int lane, int p, int j)
 {
     if (I0.key0 != ms.key || I0.fw0 != ms.fw) {
         const float4 gw = wtab ? wtab[I0.fw0] : __ldg(reinterpret_cast<const float4 *>(gwt) + I0.fw0);
@@ -361,20 +295,20 @@ __device__ __forceinline__ void sum_step_uniform(MState &ms, WarpSmem &ws, const
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int r = 8 * (k ^ j) + p;
-        P0[k] = pass_sum<T2D>(ms.M, S0, g2, r, T2D ? __shfl_sync(kFull, I0.blk, r) : 0, j);
-        P1[k] = pass_sum<T2D>(ms.M, S1, g2, r, T2D ? __shfl_sync(kFull, I1.blk, r) : 0, j);
+        P0[k] = quarter_sum(ms.M, S0, r, j);
+        P1[k] = quarter_sum(ms.M, S1, r, j);
     }
     reduce_store<DT, COMP>(P0, half_of(b, 0), sc, vis_out, lane);
     reduce_store<DT, COMP>(P1, half_of(b, 1), sc, vis_out, lane);
 }
 
-template <int DT, bool COMP, bool DIRECT, bool T2D>
+template <int DT, bool COMP, bool DIRECT>
 __global__ void __launch_bounds__(kMaxWarps * kWarp, DG_DEGRID_MIN_BLOCKS)
 degrid_kernel(const Geometry g, const void *__restrict__ subgrids, const float *__restrict__ scale,
               const double *__restrict__ uvw, const float *__restrict__ guv,
               const float *__restrict__ gwt, const Schedule sched, float2 *__restrict__ vis_out,
               DeviceStatus *__restrict__ status, const int direct_runs, const bool vec_ok,
-              const float *__restrict__ g2, const bool prefetch_uvw)
+              const bool prefetch_uvw)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     // [w table (optional)] [one WarpSmem per warp]
@@ -392,9 +326,9 @@ degrid_kernel(const Geometry g, const void *__restrict__ subgrids, const float *
     Batch bB = claimer.claim();         // rows in flight
     if (bB.n == 0)
         return;
-    Issued iB0 = issue_rows<RowStage, !T2D>(half_of(bB, 0), load_uvw(uvw, half_of(bB, 0), lane), g,
+    Issued iB0 = issue_rows<RowStage>(half_of(bB, 0), load_uvw(uvw, half_of(bB, 0), lane), g,
                                             ws.st[0][0], guv, lane, status, false);
-    Issued iB1 = issue_rows<RowStage, !T2D>(half_of(bB, 1), load_uvw(uvw, half_of(bB, 1), lane), g,
+    Issued iB1 = issue_rows<RowStage>(half_of(bB, 1), load_uvw(uvw, half_of(bB, 1), lane), g,
                                             ws.st[0][1], guv, lane, status, true);
     Batch bC = claimer.advance(bB);     // coordinates in registers
     Coords3 cC0 = load_uvw(uvw, half_of(bC, 0), lane);
@@ -419,9 +353,9 @@ degrid_kernel(const Geometry g, const void *__restrict__ subgrids, const float *
         const int sA = stage;
         bB = bC;
         if (bB.n > 0) {
-            iB0 = issue_rows<RowStage, !T2D>(half_of(bB, 0), cC0, g, ws.st[sA ^ 1][0], guv, lane, status,
+            iB0 = issue_rows<RowStage>(half_of(bB, 0), cC0, g, ws.st[sA ^ 1][0], guv, lane, status,
                                              false);
-            iB1 = issue_rows<RowStage, !T2D>(half_of(bB, 1), cC1, g, ws.st[sA ^ 1][1], guv, lane, status,
+            iB1 = issue_rows<RowStage>(half_of(bB, 1), cC1, g, ws.st[sA ^ 1][1], guv, lane, status,
                                              true);
         }
         bC = claimer.advance(bC);
@@ -442,15 +376,15 @@ degrid_kernel(const Geometry g, const void *__restrict__ subgrids, const float *
         }
         if (iA0.uniform && iA1.uniform && iA0.key0 == iA1.key0 && iA0.fw0 == iA1.fw0 &&
             bA.n == kBatchVis) {
-            sum_step_uniform<DT, COMP, T2D>(ms, ws, ws.st[sA][0], ws.st[sA][1], iA0, iA1, bA, subgrids,
-                                            base, sc, g, wtab, gwt, vis_out, vec_ok, g2, lane, p, j);
+            sum_step_uniform<DT, COMP>(ms, ws, ws.st[sA][0], ws.st[sA][1], iA0, iA1, bA, subgrids,
+                                            base, sc, g, wtab, gwt, vis_out, vec_ok, lane, p, j);
         } else {
-            sum_half<DT, COMP, DIRECT, T2D>(ms, ws, ws.st[sA][0], iA0, half_of(bA, 0), subgrids, base, sc,
-                                            g, wtab, gwt, vis_out, direct_runs, vec_ok, g2, lane, p, j);
+            sum_half<DT, COMP, DIRECT>(ms, ws, ws.st[sA][0], iA0, half_of(bA, 0), subgrids, base, sc,
+                                            g, wtab, gwt, vis_out, direct_runs, vec_ok, lane, p, j);
             if (bA.n > kBatch)
-                sum_half<DT, COMP, DIRECT, T2D>(ms, ws, ws.st[sA][1], iA1, half_of(bA, 1), subgrids, base,
-                                                sc, g, wtab, gwt, vis_out, direct_runs, vec_ok, g2, lane,
-                                                p, j);
+                sum_half<DT, COMP, DIRECT>(ms, ws, ws.st[sA][1], iA1, half_of(bA, 1), subgrids, base,
+                                                sc, g, wtab, gwt, vis_out, direct_runs, vec_ok, lane, p,
+                                                j);
         }
         __syncwarp();
         stage ^= 1;
@@ -463,20 +397,20 @@ size_t smem_bytes(const degrid_plan *p, int warps)
 }
 
 // Dynamic shared memory opened so far for a kernel instance on a device.
-template <int DT, bool COMP, bool DIRECT, bool T2D>
+template <int DT, bool COMP, bool DIRECT>
 std::atomic<size_t> &smem_record(int device)
 {
     static std::atomic<size_t> table[kMaxDevices];
     return dg_smem_record(table, device);
 }
 
-template <int DT, bool COMP, bool DIRECT, bool T2D>
+template <int DT, bool COMP, bool DIRECT>
 cudaError_t launch(degrid_plan *p, cudaStream_t st, const void *subgrids, const float *scale,
                    const double *uvw, float2 *out, const Schedule &sched, int grid_blocks)
 {
     const int threads = p->warps_per_block * kWarp;
     const size_t smem = smem_bytes(p, p->warps_per_block);
-    cudaError_t e = dg_open_smem(smem_record<DT, COMP, DIRECT, T2D>(p->device), degrid_kernel<DT, COMP, DIRECT, T2D>,
+    cudaError_t e = dg_open_smem(smem_record<DT, COMP, DIRECT>(p->device), degrid_kernel<DT, COMP, DIRECT>,
                                  smem);
     if (e != cudaSuccess)
         return e;
@@ -484,46 +418,41 @@ cudaError_t launch(degrid_plan *p, cudaStream_t st, const void *subgrids, const 
     // elements per 16 bytes
     const bool vec_ok = (reinterpret_cast<uintptr_t>(subgrids) & 15) == 0 &&
                         p->geo.nz % Storage<DT>::kQuad == 0;
-    return launch_pdl(degrid_kernel<DT, COMP, DIRECT, T2D>, dim3(grid_blocks), dim3(threads), smem, st,
+    return launch_pdl(degrid_kernel<DT, COMP, DIRECT>, dim3(grid_blocks), dim3(threads), smem, st,
                       p->geo, subgrids, scale, uvw, (const float *)p->guv, (const float *)p->gw, sched, out,
-                      p->status, p->direct_runs, vec_ok, (const float *)p->guv2, !p->host_inputs);
+                      p->status, p->direct_runs, vec_ok, !p->host_inputs);
 }
 
-template <int DT, bool COMP, bool DIRECT, bool T2D>
+template <int DT, bool COMP, bool DIRECT>
 int max_blocks(degrid_plan *p)
 {
     int n = 0;
     const size_t smem = smem_bytes(p, p->warps_per_block);
-    if (dg_open_smem(smem_record<DT, COMP, DIRECT, T2D>(p->device), degrid_kernel<DT, COMP, DIRECT, T2D>, smem) !=
+    if (dg_open_smem(smem_record<DT, COMP, DIRECT>(p->device), degrid_kernel<DT, COMP, DIRECT>, smem) !=
         cudaSuccess)
         return 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, degrid_kernel<DT, COMP, DIRECT, T2D>,
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, degrid_kernel<DT, COMP, DIRECT>,
                                                       p->warps_per_block * kWarp, smem) != cudaSuccess)
         return 1;
     return n > 0 ? n : 1;
 }
 
 // Kernel instance of a plan: storage type, compensated reduction, and one of
-// three summing forms (footprint cache; with the direct arm; 2D G_uv table).
+// two summing forms (footprint cache; with the direct arm).  Plans with a 2D
+// G_uv table have their own kernel (table2d.cu).
 template <int DT, bool COMP>
 cudaError_t launch_form(degrid_plan *p, cudaStream_t st, const void *subgrids, const float *scale,
                         const double *uvw, float2 *out, const Schedule &sched, int grid_blocks)
 {
-    if (p->guv2)
-        return launch<DT, COMP, false, true>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
     if (p->direct_runs < DG_DIRECT_RUNS_NEVER)
-        return launch<DT, COMP, true, false>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
-    return launch<DT, COMP, false, false>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
+        return launch<DT, COMP, true>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
+    return launch<DT, COMP, false>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
 }
 
 template <int DT, bool COMP>
 int max_blocks_form(degrid_plan *p)
 {
-    if (p->guv2)
-        return max_blocks<DT, COMP, false, true>(p);
-    if (p->direct_runs < DG_DIRECT_RUNS_NEVER)
-        return max_blocks<DT, COMP, true, false>(p);
-    return max_blocks<DT, COMP, false, false>(p);
+    return p->direct_runs < DG_DIRECT_RUNS_NEVER ? max_blocks<DT, COMP, true>(p) : max_blocks<DT, COMP, false>(p);
 }
 
 template <int DT>
@@ -549,6 +478,8 @@ cudaError_t dg_launch_degrid(degrid_plan *p, cudaStream_t st, const void *subgri
 {
     using namespace dg;
     (void)vis_offsets;
+    if (p->guv2)
+        return dg_launch_degrid_2d(p, st, subgrids, scale, uvw, out_f, grid_blocks);
     Schedule sched{p->chunks, p->n_chunks, p->work_counter};
     float2 *out = reinterpret_cast<float2 *>(out_f);
     switch (p->dtype) {
@@ -565,6 +496,8 @@ cudaError_t dg_launch_degrid(degrid_plan *p, cudaStream_t st, const void *subgri
 int dg_max_blocks_per_sm_degrid(degrid_plan *p)
 {
     using namespace dg;
+    if (p->guv2)
+        return dg_max_blocks_per_sm_degrid_2d(p);
     switch (p->dtype) {
     case DG_C64: return max_blocks_dt<DG_C64>(p);
     case DG_C32_F16: return max_blocks_dt<DG_C32_F16>(p);

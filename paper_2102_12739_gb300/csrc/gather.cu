@@ -39,6 +39,7 @@
 //
 // Requirements (checked by the host): nz = 4, a separable G_uv table, a
 // 16-byte aligned subgrid stack.
+#include "footprint.cuh"
 #include "pipeline.cuh"
 #include "tma.cuh"
 
@@ -207,14 +208,6 @@ __device__ __forceinline__ void column(const GatherSlot<DT> &sl, int v, int b, i
     }
 }
 
-__device__ __forceinline__ float two_sum_g(float a, float b, float &e)
-{
-    const float s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    return s;
-}
-
 // Sums the stage in `sl` and stores its visibilities.
 template <int DT, bool COMP>
 __device__ __forceinline__ void sum_stage(const GatherSlot<DT> &sl, const float4 *wtab,
@@ -251,10 +244,10 @@ __device__ __forceinline__ void sum_stage(const GatherSlot<DT> &sl, const float4
     float2 V;
     if (COMP) {
         float2 e0, e;
-        const float2 S = make_float2(two_sum_g(Q.x, __shfl_xor_sync(kFull, Q.x, 4), e0.x),
-                                     two_sum_g(Q.y, __shfl_xor_sync(kFull, Q.y, 4), e0.y));
-        V.x = two_sum_g(S.x, __shfl_xor_sync(kFull, S.x, 2), e.x);
-        V.y = two_sum_g(S.y, __shfl_xor_sync(kFull, S.y, 2), e.y);
+        const float2 S = make_float2(two_sum(Q.x, __shfl_xor_sync(kFull, Q.x, 4), e0.x),
+                                     two_sum(Q.y, __shfl_xor_sync(kFull, Q.y, 4), e0.y));
+        V.x = two_sum(S.x, __shfl_xor_sync(kFull, S.x, 2), e.x);
+        V.y = two_sum(S.y, __shfl_xor_sync(kFull, S.y, 2), e.y);
         e.x += e0.x + __shfl_xor_sync(kFull, e0.x, 2);
         e.y += e0.y + __shfl_xor_sync(kFull, e0.y, 2);
         V.x += e.x;

@@ -357,5 +357,9 @@ cudaError_t dg_launch_scatter(degrid_plan *p, cudaStream_t st, int n_subgrids, c
 int dg_scatter_warps();                         // warps per CTA of the scattered gridding kernel
 bool dg_gather_supported(const degrid_plan *p);
 int dg_max_blocks_per_sm_degrid(degrid_plan *p);
+// plans with a 2D G_uv table (called through the two above)
+cudaError_t dg_launch_degrid_2d(degrid_plan *p, cudaStream_t st, const void *subgrids, const float *scale,
+                                const double *uvw, float *vis_out, int grid_blocks);
+int dg_max_blocks_per_sm_degrid_2d(degrid_plan *p);
 int dg_max_warps_per_block();        // largest warps_per_block the kernels are built for
 int dg_max_blocks_per_sm_adjoint(degrid_plan *p);

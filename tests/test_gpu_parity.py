@@ -1108,3 +1108,34 @@ def test_packing_every_form_bitwise(dtype, S, elems, shift):
     q = q.to(codes.dtype)
     same = (codes == q) | (codes.isnan() & q.isnan())
     assert bool(same.all())
+
+
+@pytest.mark.parametrize("dtype,comp", [("c64", False), ("f16", True), ("bf16", False)])
+@pytest.mark.parametrize("nz", [4, 5])
+def test_table2d_steps_of_many_runs(dtype, comp, nz):
+    # steps with 1, 2, 7, 8, 9, 17 and 32 runs of equal footprint and w row
+    # (a warp holds 8 footprints), runs that continue over steps and come
+    # back, invalid visibilities inside runs, ragged ends
+    d = dev()
+    shape = (40, 48, nz)
+    G2 = synth.default_table_2d(16)
+    rng = np.random.default_rng(nz)
+    ends = []
+    for n_runs in (1, 1, 2, 7, 8, 9, 17, 32, 1, 3):
+        p = np.stack([rng.uniform(4, 40, n_runs), rng.uniform(4, 32, n_runs), rng.uniform(1.0, nz - 2.01, n_runs)], 1)
+        ends.append(p[np.sort(rng.integers(0, n_runs, 32))] if n_runs not in (1, 32) else p[np.arange(32) % n_runs])
+    uvw = np.concatenate(ends + [ends[0][:9]])
+    uvw[[5, 70, 71, 133, 200]] = [[np.nan, 9, 1.5], [1e9, 9, 1.5], [-3, 9, 1.5], [9, 1e300, 1.5], [9, 9, 77.0]]
+    sub = torch.from_numpy(synth.subgrid_stack(1, shape=shape)).to(d)
+    codes, scale = (sub, None) if dtype == "c64" else dg.pack_subgrids(sub, dtype)
+    stored = sub.cpu().numpy().astype(np.complex128)
+    if dtype != "c64":
+        q = codes.float().cpu().numpy().astype(np.float64) * float(scale[0])
+        stored = q[..., 0] + 1j * q[..., 1]
+    offs = np.array([0, len(uvw)])
+    ref, bad = oracle.degrid_2d(G2, synth.default_tables()[1], stored, uvw, offs)
+    with dg.DegridPlan(shape=shape, dtype=dtype, device=d, g_uv2=G2, compensated=comp) as p:
+        got = p.degrid(codes, torch.from_numpy(uvw).to(d), torch.from_numpy(offs).to(d), scale=scale).cpu().numpy()
+        assert p.status() == bad == 5
+    assert np.linalg.norm(got - ref) <= 2e-6 * np.linalg.norm(ref)
+    assert np.all(got[[5, 70, 71, 133, 200]] == 0)
