@@ -25,7 +25,7 @@ LIB_PATH = os.path.join(OUT_DIR, "libdegrid.so")
 
 SOURCES = ["api.cu", "schedule.cu", "degrid.cu", "table2d.cu", "adjoint.cu", "aux_kernels.cu", "noalloc.cu",
            "host_exec.cu", "peak.cu",
-           "gather.cu", "scatter.cu", "predict.cu", "predict_fft.cu"]
+           "gather.cu", "scatter.cu", "bins.cu", "tiled_degrid.cu", "tiled_grid.cu", "predict.cu", "predict_fft.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2",
               "-I", INCLUDE, "-I", CSRC]

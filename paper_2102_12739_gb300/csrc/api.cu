@@ -7,6 +7,7 @@
 #include <new>
 #include <vector>
 
+#include "bins.cuh"
 #include "internal.cuh"
 
 cudaError_t dg_launch_pack(cudaStream_t st, dg_dtype dtype, int n_subgrids, int64_t elems,
@@ -79,6 +80,7 @@ void free_plan_buffers(degrid_plan *p)
 {
     free_events(p);
     dg_free_host_exec(p);
+    dg_bins_free(p);
     cudaFree(p->guv);
     cudaFree(p->guv2);
     cudaFree(p->gw);
@@ -141,7 +143,8 @@ dg_status ensure_capacity(degrid_plan *p, int S, int64_t n_vis, int chunk)
     if (need_chunks > 0x7fffffff)
         return DG_ERR_ARG;
     if (S > p->cap_subgrids) {
-        cudaDeviceSynchronize();
+        if (p->prefix)
+            cudaDeviceSynchronize();
         cudaFree(p->prefix);
         p->prefix = nullptr;
         p->cap_subgrids = 0;
@@ -151,7 +154,8 @@ dg_status ensure_capacity(degrid_plan *p, int S, int64_t n_vis, int chunk)
         p->cap_subgrids = S;
     }
     if (need_chunks > p->cap_chunks) {
-        cudaDeviceSynchronize();
+        if (p->chunks)
+            cudaDeviceSynchronize();
         cudaFree(p->chunks);
         p->chunks = nullptr;
         p->cap_chunks = 0;
@@ -190,6 +194,13 @@ struct KernelTimer {
 bool tma_rows_fit(const degrid_plan *p, int n_subgrids)
 {
     return (int64_t)n_subgrids * p->geo.ny <= (int64_t)0x7fffffff;
+}
+
+// Whether a call of a plan with the gather setting goes by tiles: worth it,
+// and the workspace fits (or can grow now).
+bool tiled(degrid_plan *p, cudaStream_t st, dg::TileShape shape, int n_subgrids, int64_t n_vis)
+{
+    return p->gather && dg_bins_worth(p, shape, n_subgrids, n_vis) && dg_bins_reserve(p, st, shape, n_subgrids, n_vis);
 }
 
 // Persistent grid: the resident CTAs of every SM, but no more CTAs than
@@ -561,11 +572,20 @@ dg_status degrid_execute(degrid_plan_t p, void *stream, int n_subgrids, const vo
     DeviceGuard guard(p->device);
     if (!guard.ok)
         return DG_ERR_CUDA;
+    cudaStream_t s = (cudaStream_t)stream;
     const int chunk = call_chunk(p, n_vis);
     dg_status st = ensure_capacity(p, n_subgrids, n_vis, chunk);
     if (st != DG_OK)
         return st;
-    cudaStream_t s = (cudaStream_t)stream;
+    if (tiled(p, s, kDegridTile, n_subgrids, n_vis)) {
+        KernelTimer timer(p, s);
+        dg::Bins bins;
+        cudaError_t e = dg_bins_sort(p, s, kDegridTile, n_subgrids, n_vis, uvw, vis_offsets, vis_out, &bins);
+        if (e == cudaSuccess)
+            e = dg_launch_tiled_degrid(p, s, bins, p->bins->cap_items, subgrids, n_subgrids, subgrid_scale, vis_out);
+        timer.stop();
+        return from_cuda(e);
+    }
     cudaError_t e = dg::launch_schedule(s, vis_offsets, n_subgrids, n_vis, chunk, dg_small_items(chunk),
                                         p->prefix, p->n_chunks, p->chunks, p->cap_chunks, p->work_counter,
                                         p->status);
@@ -616,6 +636,15 @@ dg_status grid_adjoint_execute(degrid_plan_t p, void *stream, int n_subgrids, co
     dg_status st = ensure_capacity(p, n_subgrids, n_vis, chunk);
     if (st != DG_OK)
         return st;
+    if (aligned(sub_out, 16) && tiled(p, s, kGridTile, n_subgrids, n_vis)) {
+        KernelTimer timer(p, s);
+        dg::Bins bins;
+        cudaError_t e = dg_bins_sort(p, s, kGridTile, n_subgrids, n_vis, uvw, vis_offsets, nullptr, &bins);
+        if (e == cudaSuccess)
+            e = dg_launch_tiled_grid(p, s, bins, p->bins->cap_items, n_subgrids, vis_in, sub_out);
+        timer.stop();
+        return from_cuda(e);
+    }
     cudaError_t e = dg::launch_schedule(s, vis_offsets, n_subgrids, n_vis, chunk, dg_small_items(chunk),
                                         p->prefix, p->n_chunks, p->chunks, p->cap_chunks, p->work_counter,
                                         p->status);

@@ -254,6 +254,7 @@ struct degrid_plan {
     int host_inputs;            // set during such a call: the kernel's inputs are in host memory
     int max_blocks_degrid;      // occupancy results, 0 = not computed yet
     int max_blocks_adjoint;
+    struct dg_bins *bins;       // workspace of the calls sorted by tile (bins.cu), lazily
     struct dg_host_exec *hostx; // streams and staging of degrid_execute_host (host_exec.cu), lazily
     int n_slots;                // timing event pairs (0 = timing off)
     long long timed_launches;

@@ -82,13 +82,11 @@ __device__ __forceinline__ void fence_mbarrier_init()
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-// A 2D tensor map (host side): dim0 x dim1 elements of type `type`, rows
-// `stride` bytes apart, boxes of box0 x box1 elements, no swizzle.
-inline cudaError_t encode_2d(CUtensorMap *map, void *base, CUtensorMapDataType type, uint64_t dim0,
-                             uint64_t dim1, uint64_t stride, uint32_t box0, uint32_t box1)
+// cuTensorMapEncodeTiled, looked up once (a function-local static:
+// initialised once, also under concurrent first calls from several host
+// threads); nullptr if the driver has none.
+inline PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
 {
-    // looked up once (a function-local static: initialised once, also under
-    // concurrent first calls from several host threads)
     static const PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
         cudaDriverEntryPointQueryResult q;
         void *fn = nullptr;
@@ -98,16 +96,52 @@ inline cudaError_t encode_2d(CUtensorMap *map, void *base, CUtensorMapDataType t
                    ? reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn)
                    : nullptr;
     }();
+    return encode;
+}
+
+// A tensor map of `rank` dimensions (host side), no swizzle: strides in bytes
+// of dimensions 1 and up.
+inline cudaError_t encode_map(CUtensorMap *map, void *base, CUtensorMapDataType type, int rank, const uint64_t *dim,
+                              const uint64_t *stride, const uint32_t *box)
+{
+    const PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
     if (!encode)
         return cudaErrorNotSupported;
-    const cuuint64_t dims[2] = {(cuuint64_t)dim0, (cuuint64_t)dim1};
-    const cuuint64_t strides[1] = {(cuuint64_t)stride};
-    const cuuint32_t box[2] = {(cuuint32_t)box0, (cuuint32_t)box1};
-    const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = encode(map, type, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    cuuint64_t dims[3], strides[2];
+    cuuint32_t boxes[3];
+    const cuuint32_t estr[3] = {1, 1, 1};
+    for (int k = 0; k < rank; ++k) {
+        dims[k] = dim[k];
+        boxes[k] = box[k];
+        if (k > 0)
+            strides[k - 1] = stride[k - 1];
+    }
+    const CUresult r = encode(map, type, (cuuint32_t)rank, base, dims, strides, boxes, estr,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                              CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// dim0 x dim1 elements of type `type`, rows `stride` bytes apart, boxes of
+// box0 x box1 elements.
+inline cudaError_t encode_2d(CUtensorMap *map, void *base, CUtensorMapDataType type, uint64_t dim0,
+                             uint64_t dim1, uint64_t stride, uint32_t box0, uint32_t box1)
+{
+    const uint64_t dim[2] = {dim0, dim1};
+    const uint32_t box[2] = {box0, box1};
+    return encode_map(map, base, type, 2, dim, &stride, box);
+}
+
+// A stack of dim2 planes of dim1 rows of dim0 elements of elem_bytes each,
+// contiguous; boxes of box0 x box1 elements of one plane, clipped (reads:
+// filled with zeros) at the edges of the plane.
+inline cudaError_t encode_3d(CUtensorMap *map, void *base, CUtensorMapDataType type, uint64_t dim0, uint64_t dim1,
+                             uint64_t dim2, uint64_t elem_bytes, uint32_t box0, uint32_t box1)
+{
+    const uint64_t dim[3] = {dim0, dim1, dim2};
+    const uint64_t stride[2] = {dim0 * elem_bytes, dim0 * dim1 * elem_bytes};
+    const uint32_t box[3] = {box0, box1, 1};
+    return encode_map(map, base, type, 3, dim, stride, box);
 }
 
 // The tensor map of a stack of n_subgrids subgrids (host side), with boxes

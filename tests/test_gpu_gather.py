@@ -173,3 +173,77 @@ def test_scatter_gridding_full_size_and_dot_product():
     assert abs(lhs - rhs) <= 1e-5 * abs(lhs)
     ref, _ = oracle.grid(G_UV, G_W, synth.SUBGRID_SHAPE, w.n_subgrids, w.uvw, w.vis_offsets, y)
     assert rel_l2(gnp, ref) <= TOL["c64"]
+
+
+TILED = [   # shape, counts, kind: enough visibilities per tile for the tile kernels
+    ((48, 48, 4), [250000], "scatter"),
+    ((71, 135, 4), [40000, 0, 170001, 33], "scatter"),         # tiles end inside and at the last start
+    ((103, 87, 4), [220000, 1], "line"),                        # dense: whole warps in one tile
+    ((512, 512, 4), [260000, 1], "mixed"),
+]
+
+
+@pytest.mark.parametrize("shape,counts,kind", TILED)
+@pytest.mark.parametrize("dtype,comp", [("c64", False), ("f16", True), ("bf16", False)])
+def test_tiled_degridding_is_bitwise_the_cached_path(shape, counts, kind, dtype, comp):
+    d = dev()
+    w = small_workload(counts, kind=kind, shape=shape, seed=91)
+    uvw_np = w.uvw.copy()
+    bad = [0, 31, 32, 1777, len(uvw_np) - 1]
+    uvw_np[bad] = [[np.nan, 9, 1.5], [1e9, 9, 1.5], [9, -2, 1.5], [9, 9, 77.0], [3.4, 1e300, 1.2]]
+    # the corners of the valid box: first and last start of the first and last tile
+    ny, nx, _ = shape
+    uvw_np[100:104] = [[3, 3, 1.0], [nx - 5 + 0.999, 3, 1.5], [3, ny - 5 + 0.999, 1.99], [nx - 5, ny - 5, 1.0]]
+    sub = torch.from_numpy(synth.subgrid_stack(len(counts), shape=shape)).to(d)
+    codes, scale = (sub, None) if dtype == "c64" else dg.pack_subgrids(sub, dtype)
+    uvw, offs = torch.from_numpy(uvw_np).to(d), torch.from_numpy(w.vis_offsets).to(d)
+    outs = []
+    for gather in (False, True):
+        with dg.DegridPlan(shape=shape, dtype=dtype, device=d, compensated=comp, gather=gather) as p:
+            out = torch.full((w.n_vis,), float("nan"), dtype=torch.complex64, device=d)
+            outs.append(p.degrid(codes, uvw, offs, scale=scale, out=out).cpu().numpy())
+            assert p.status() == len(bad)
+    np.testing.assert_array_equal(outs[0].view(np.uint64), outs[1].view(np.uint64))
+
+
+@pytest.mark.parametrize("shape,counts,kind", TILED)
+def test_tiled_gridding_matches_oracle(shape, counts, kind):
+    d = dev()
+    w = small_workload(counts, kind=kind, shape=shape, seed=92)
+    uvw_np = w.uvw.copy()
+    uvw_np[[5, 1234]] = [[np.inf, 9, 1.5], [9, 9, -1.0]]
+    y = synth.adjoint_vis(w.n_vis)
+    ref, bad = oracle.grid(G_UV, G_W, shape, len(counts), uvw_np, w.vis_offsets, y)
+    assert bad == 2
+    with dg.DegridPlan(shape=shape, device=d, gather=True) as p:
+        args = (torch.from_numpy(y).to(d), torch.from_numpy(uvw_np).to(d), torch.from_numpy(w.vis_offsets).to(d),
+                len(counts))
+        out = p.grid(*args)
+        assert p.status() == 2
+        assert rel_l2(out.cpu().numpy(), ref) <= 2e-6
+        p.grid(*args, out=out, accumulate=True)
+        assert rel_l2(out.cpu().numpy(), 2 * ref) <= 2e-6
+        assert p.status() == 2
+
+
+def test_a_captured_call_larger_than_the_tiles_workspace():
+    # a plan that has only seen few visibilities cannot grow its workspace
+    # inside a capture: the call is captured through the gather kernel
+    d = dev()
+    shape = (64, 64, 4)
+    w = small_workload([300000], kind="scatter", shape=shape, seed=93)
+    sub = torch.from_numpy(synth.subgrid_stack(1, shape=shape)).to(d)
+    uvw, offs = torch.from_numpy(w.uvw).to(d), torch.from_numpy(w.vis_offsets).to(d)
+    out = torch.zeros(w.n_vis, dtype=torch.complex64, device=d)
+    with dg.DegridPlan(shape=shape, device=d) as p:
+        p.degrid(sub, uvw, offs)                        # the chunk table, without tiles
+        p.set_gather(True)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            p.degrid(sub, uvw, offs, out=out)
+        g.replay()
+        torch.cuda.synchronize()
+        first = out.cpu().numpy()
+        second = p.degrid(sub, uvw, offs).cpu().numpy()         # by tiles
+        assert p.status() == 0
+    np.testing.assert_array_equal(first.view(np.uint64), second.view(np.uint64))
