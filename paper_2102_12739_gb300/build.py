@@ -23,7 +23,7 @@ INCLUDE = os.path.join(ROOT, "include")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB_PATH = os.path.join(OUT_DIR, "libdegrid.so")
 
-SOURCES = ["api.cu", "schedule.cu", "degrid.cu", "table2d.cu", "adjoint.cu", "aux_kernels.cu", "noalloc.cu",
+SOURCES = ["api.cu", "schedule.cu", "degrid.cu", "direct.cu", "table2d.cu", "adjoint.cu", "aux_kernels.cu", "noalloc.cu",
            "host_exec.cu", "peak.cu",
            "gather.cu", "scatter.cu", "bins.cu", "tiled_degrid.cu", "tiled_grid.cu", "predict.cu", "predict_fft.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

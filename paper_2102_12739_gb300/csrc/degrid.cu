@@ -2,393 +2,462 @@
 // variants), re-designed for sm_103a.
 //
 // Work decomposition (pipeline.cuh).  A persistent grid of warps walks chunks
-// of consecutive visibilities of one subgrid in steps of 64 (two halves of
-// 32, which amortises the per-step bookkeeping and gives every lane two
-// independent coordinates to snap).  Three stages overlap across consecutive
-// steps of a warp:
-//  1. the FP64 coordinates of step n + 2 are loaded into registers (and the
-//     next chunk's are prefetched into L2 when its descriptor arrives);
-//  2. step n + 1 is snapped (one visibility per lane and half) and its g_u and
-//     g_v rows are copied into the warp's shared-memory stage with cp.async;
-//  3. step n is summed from the stage that arrived, one half after the other.
+// of consecutive visibilities of one subgrid in steps of 64: lane i owns
+// visibilities i and i + 32 of the step from the coordinates to the store.
+// Per step a warp
+//  1. snaps the coordinates of the next step (loaded one step before; the
+//     next chunk's are prefetched into L2 when its descriptor arrives), while
+//     the table rows of the current step are on their way;
+//  2. loads the coordinates of the step after that;
+//  3. builds the footprints M it does not hold yet, sums and stores;
+//  4. starts the copies (cp.async) of the next step's g_u and g_v rows into
+//     the warp's shared-memory stage, two lanes per 32-byte row.
 //
 // Footprint sum.  The separable weights let the 8 x 8 x 4 sum be taken in
 // three contractions,
 //     V = sum_b g_v[b] sum_a g_u[a] M[b][a],   M[b][a] = sum_c g_w[c] s[y0+b][x0+a][z0+c],
 // and M depends only on the footprint start and the w-kernel row.  On a dense
 // list hundreds of consecutive visibilities share both (the reuse the paper
-// notes for D1), so M is computed once per run and each visibility then costs
-// 72 complex x real products instead of 256.
+// notes for D1), so M is computed once per run, by the whole warp, into one
+// of the warp's shared-memory slots, and each visibility then costs 72
+// complex x real products instead of 256.  Every lane reads M from shared
+// memory: lanes of one run read the same address (a broadcast), and when both
+// visibilities of every lane share a run, one read serves two products.
+// Slots start 16 bytes further into the 128-byte bank line than the slot
+// before, so lanes of several runs read different banks: a step that holds up
+// to kSlots runs is built and summed in one pass.
 //
-// Lanes.  Four lanes share a visibility: lane 8j + p (j = 0..3, p = 0..7)
-// holds the rows M[2j][0..7] and M[2j+1][0..7] of the footprint in 32
-// registers and, for a visibility r, forms
-// sum_{b = 2j, 2j+1} g_v[b] sum_a g_u[a] M[b][a] (36 FP32 operations).  A
-// half takes four passes; in pass k lane 8j + p works on visibility
-// 8 (k ^ j) + p, an order chosen so that the two exchange steps of the
-// reduction move the same pass slots on every lane (no selects): lane xor 16
-// adds slots 2, 3 to 0, 1, then lane xor 8 adds slot 1 to slot 0, and lane
-// 8j + p ends with visibility 8j + p, so the warp writes its 32 results into
-// one contiguous 256-byte segment in lane order.  The 8 lanes of one 128-bit
-// shared-memory wavefront read 8 consecutive rows of the stage, which its
-// half-swapped layout places in 8 different bank groups.  M is built by the
-// whole warp (two entries per lane) into shared memory and read back by rows;
-// a half whose 32 visibilities share one footprint and w row needs no checks,
-// and any other half is summed once per distinct (footprint, w row) it holds,
-// every lane keeping the pass that matches its own visibility.
-// The products use packed FFMA2 on (re, im) pairs with a duplicated real
-// weight: bitwise the same as two scalar FMAs, in half the instructions
-// (11.2 instead of 12.7 warp instructions per visibility on dense lines).
+// Every operation and its order are those of the gather, tile and 2D-table
+// kernels, so all agree bit for bit.
+//
+// What bounds it.  16M visibilities on 64 subgrids' lines take 211 us, 260
+// cycles per SM and 64 visibilities.  Of those the requests to L1 and L2 take
+// about 175 (128 table rows at 1.06 cycles each, measured in isolation,
+// whatever the copy; the coordinates and the output), the load/store data
+// path 165, the six FP64-to-int32 conversions of the snap 96 (16 cycles per
+// warp instruction), the packed FMAs 76; 16 warps per SM overlap them at 62%.
+// Measured and slower: the rows loaded into registers by each lane (249 us:
+// a data-path cycle per row), two row stages (278: the copies queue up before
+// the coordinate loads), coordinates copied to shared memory (225), 24 warps
+// with 80 registers (242).
+//
+// Four lanes per visibility, each with two rows of M in registers, took 222
+// us here and summed a step with several runs once per run and eight
+// visibilities: 14M visibilities on 96 subgrids' lines and arcs of uneven
+// length took 284 us, and take 237.
+#include <type_traits>
+
 #include "footprint.cuh"
 #include "pipeline.cuh"
 
 namespace dg {
 namespace {
 
-#ifndef DG_DEGRID_MIN_BLOCKS
-#define DG_DEGRID_MIN_BLOCKS 2   // resident CTAs per SM the register budget is sized for
-#endif
-
 constexpr int kMaxWarps = 8;                // per CTA
-constexpr int kBatchVis = 2 * kBatch;       // visibilities per pipeline step (two halves)
-struct alignas(128) WarpSmem {
-    RowStage st[2][2];          // [stage][half]
-    float2 m[8][8];             // M[b][a] of the footprint being built
-    float2 part[4][kWarp];      // per-pass partials on the mixed path
+constexpr int kStepVis = 2 * kBatch;        // visibilities per pipeline step: two per lane
+constexpr int kSlots = 8;                   // footprints a warp holds (a power of two)
+
+// M[b][a] of one footprint; the padding moves the next slot by one 16-byte
+// bank group.
+struct alignas(16) MSlot {
+    float2 m[kUV][kUV];
+    float2 pad[2];
 };
+
+struct alignas(128) WarpSmem {
+    RowStage st[2];             // [half]
+    MSlot slot[kSlots];
+};
+
+// A step: subgrid, visibilities left in its chunk from here on (0: no work
+// left), and where this lane's first visibility is read and written.
+struct Step {
+    int s, n;
+    const double *uvw;
+    float2 *out;
+};
+
+// Steps of the chunks a warp claims.
+struct Steps {
+    ClaimerT<kStepVis> claimer;
+    const double *uvw;          // this lane's offset included
+    float2 *out;
+
+    __device__ Step claim()
+    {
+        const Batch b = claimer.claim();
+        return Step{b.s, (int)(b.end - b.b0), uvw + 3 * b.b0, out + b.b0};
+    }
+
+    __device__ Step advance(const Step &p)
+    {
+        if (p.n == 0)
+            return p;
+        if (p.n <= kStepVis)
+            return claim();
+        return Step{p.s, p.n - kStepVis, p.uvw + 3 * kStepVis, p.out + kStepVis};
+    }
+};
+
+// Coordinates of the lane's two visibilities (zeros past the end).
+__device__ __forceinline__ void load_coords(Coords3 (&c)[2], const Step &p, int lane)
+{
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        c[h] = Coords3{0.0, 0.0, 0.0};
+        if (lane + kBatch * h < p.n) {
+            c[h].u = __ldg(p.uvw + 3 * kBatch * h);
+            c[h].v = __ldg(p.uvw + 3 * kBatch * h + 1);
+            c[h].w = __ldg(p.uvw + 3 * kBatch * h + 2);
+        }
+    }
+}
 
 // ---- the factored sum -------------------------------------------------------
 
-// M[2j + i][a] for i = 0, 1 and a = 0..7 of footprint `key` (subgrid at
-// `base`) with w row gw: lane (a = lane & 7, b = lane >> 3 and b + 4)
-// computes two entries into shared memory, then every lane reads its rows.
-template <int DT>
-__device__ __forceinline__ void build_rows(float2 (&M)[2][8], float2 (&mbuf)[8][8], const void *sub,
-                                           int64_t base, int key, const float4 &gw, const Geometry &g,
-                                           bool vec_ok, int lane, int j)
-{
-    const int a = lane & 7, b = lane >> 3;
-    const int64_t col = base + key + (int64_t)a * g.nz;
-    const bool vec = vec_footprint<DT>(vec_ok, key);
-    __syncwarp();                               // previous read-back done
-#pragma unroll
-    for (int k = 0; k < 2; ++k)
-        mbuf[b + 4 * k][a] = footprint_point<DT>(sub, col + (int64_t)(b + 4 * k) * g.row_stride, gw, vec);
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-#pragma unroll
-        for (int a2 = 0; a2 < 8; a2 += 2) {
-            const float4 t = *reinterpret_cast<const float4 *>(&mbuf[2 * j + i][a2]);
-            M[i][a2] = make_float2(t.x, t.y);
-            M[i][a2 + 1] = make_float2(t.z, t.w);
-        }
-    }
-}
-
-// This lane's quarter of visibility r: sum_{i} g_v[2j + i] sum_a g_u[a] M[i][a].
-__device__ __forceinline__ float2 quarter_sum(const float2 (&M)[2][8], const RowStage &S, int r, int j)
-{
-    const float4 u0 = S.u[r][row_half(r, 0)];
-    const float4 u1 = S.u[r][row_half(r, 1)];
-    const float2 v = reinterpret_cast<const float2 *>(&S.v[r][row_half(r, j >> 1)])[j & 1];
-    const float gu[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-    // complex x real products as packed pairs (re, im) * (g, g): one FFMA2
-    // per product, each half rounded exactly as a scalar FMA
-    float2 t0 = __fmul2_rn(M[0][0], make_float2(gu[0], gu[0]));
-    float2 t1 = __fmul2_rn(M[1][0], make_float2(gu[0], gu[0]));
-#pragma unroll
-    for (int a = 1; a < 8; ++a) {
-        t0 = __ffma2_rn(M[0][a], make_float2(gu[a], gu[a]), t0);
-        t1 = __ffma2_rn(M[1][a], make_float2(gu[a], gu[a]), t1);
-    }
-    return __ffma2_rn(t1, make_float2(v.y, v.y), __fmul2_rn(t0, make_float2(v.x, v.x)));
-}
-
-// Direct arm: this lane's quarter of visibility r (footprint `key`, w row gw)
-// from the subgrid itself, M's two rows formed on the fly; the same
-// operations in the same order as build_rows followed by quarter_sum.
-template <int DT>
-__device__ __forceinline__ float2 quarter_sum_direct(const void *sub, int64_t base, int key,
-                                                    const float4 &gw, const RowStage &S, int r, int j,
-                                                    const Geometry &g, bool vec_ok)
-{
-    const bool vec = vec_footprint<DT>(vec_ok, key);
-    const float4 u0 = S.u[r][row_half(r, 0)];
-    const float4 u1 = S.u[r][row_half(r, 1)];
-    const float2 v = reinterpret_cast<const float2 *>(&S.v[r][row_half(r, j >> 1)])[j & 1];
-    const float gu[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-    const int64_t e0 = base + key + (int64_t)(2 * j) * g.row_stride, e1 = e0 + g.row_stride;
-    float2 m0[8], m1[8];
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {             // all loads issued before the sums
-        m0[a] = footprint_point<DT>(sub, e0 + (int64_t)a * g.nz, gw, vec);
-        m1[a] = footprint_point<DT>(sub, e1 + (int64_t)a * g.nz, gw, vec);
-    }
-    float2 t0 = __fmul2_rn(m0[0], make_float2(gu[0], gu[0]));
-    float2 t1 = __fmul2_rn(m1[0], make_float2(gu[0], gu[0]));
-#pragma unroll
-    for (int a = 1; a < 8; ++a) {
-        t0 = __ffma2_rn(m0[a], make_float2(gu[a], gu[a]), t0);
-        t1 = __ffma2_rn(m1[a], make_float2(gu[a], gu[a]), t1);
-    }
-    return __ffma2_rn(t1, make_float2(v.y, v.y), __fmul2_rn(t0, make_float2(v.x, v.x)));
-}
-
-// State of the cached footprint matrix: rows 2j, 2j + 1 of M for (key, fw)
-// in the subgrid at `base` (key -2: none).
-struct MState {
-    float2 M[2][8];
-    int key, fw;
+// What the M builds of a warp need besides the footprint.
+struct BuildArgs {
+    const void *subgrids;
+    const float4 *wtab;             // w table in shared memory, or nullptr
+    const float *gwt;               // w table in global memory
+    bool vec_ok;
+    int lane;
 };
 
-// Sums one half batch (32 visibilities, stage S, issued info I), reduces the
-// four lane partials and stores visibility `lane` of the half.
-// Reduces the four pass slots of every lane to visibility `lane` of the half
-// and stores it (times the subgrid's scale for FP16/BF16 storage).
-template <int DT, bool COMP>
-__device__ __forceinline__ void reduce_store(float2 (&P)[4], const Batch &h, float sc,
-                                             float2 *__restrict__ vis_out, int lane)
+__device__ __forceinline__ float4 w_row(const BuildArgs &A, int fw)
 {
-    // lane xor 16 (j ^ 2) brings slots 2, 3 onto 0, 1; lane xor 8 (j ^ 1)
-    // brings slot 1 onto 0
-    float2 V;
-    if (COMP) {
-        // the same three additions as error-free sums; the four rounding
-        // errors are summed and added back once
-        float2 e0, e1, e;
-        P[0].x = two_sum(P[0].x, __shfl_xor_sync(kFull, P[2].x, 16), e0.x);
-        P[0].y = two_sum(P[0].y, __shfl_xor_sync(kFull, P[2].y, 16), e0.y);
-        P[1].x = two_sum(P[1].x, __shfl_xor_sync(kFull, P[3].x, 16), e1.x);
-        P[1].y = two_sum(P[1].y, __shfl_xor_sync(kFull, P[3].y, 16), e1.y);
-        V.x = two_sum(P[0].x, __shfl_xor_sync(kFull, P[1].x, 8), e.x);
-        V.y = two_sum(P[0].y, __shfl_xor_sync(kFull, P[1].y, 8), e.y);
-        e.x += e0.x + __shfl_xor_sync(kFull, e1.x, 8);
-        e.y += e0.y + __shfl_xor_sync(kFull, e1.y, 8);
-        V.x += e.x;
-        V.y += e.y;
-    } else {
-        P[0].x += __shfl_xor_sync(kFull, P[2].x, 16);
-        P[0].y += __shfl_xor_sync(kFull, P[2].y, 16);
-        P[1].x += __shfl_xor_sync(kFull, P[3].x, 16);
-        P[1].y += __shfl_xor_sync(kFull, P[3].y, 16);
-        V.x = P[0].x + __shfl_xor_sync(kFull, P[1].x, 8);
-        V.y = P[0].y + __shfl_xor_sync(kFull, P[1].y, 8);
-    }
-    if (DT != DG_C64)
-        V = __fmul2_rn(V, make_float2(sc, sc));
-    if (lane < h.n)                     // lane 8j + p holds visibility 8j + p of the half
-        vis_out[h.b0 + lane] = V;
+    return A.wtab ? A.wtab[fw] : __ldg(reinterpret_cast<const float4 *>(A.gwt) + fw);
 }
 
-
-template <int DT, bool COMP, bool DIRECT>
-__device__ __forceinline__ void sum_half(MState &ms, WarpSmem &ws, const RowStage &S, const Issued &I,
-                                         const Batch &h, const void *__restrict__ subgrids, int64_t base,
-                                         float sc, const Geometry &g, const float4 *wtab,
-                                         const float *__restrict__ gwt, float2 *__restrict__ vis_out,
-                                         int direct_runs, bool vec_ok, int lane, int p, int j)
+// This lane's two points of M for footprint `key`, w row fw of the subgrid at
+// element `base`: column lane & 7 of rows lane >> 3 and (lane >> 3) + 4.
+template <int DT>
+__device__ __forceinline__ void build_points(float2 (&m)[2], int64_t base, int key, int fw, const Geometry &g,
+                                             const BuildArgs &A)
 {
-    float2 P[4];                        // pass k: this lane's quarter of visibility 8 (k ^ j) + p
-    if (I.uniform) {
-        if (I.key0 != ms.key || I.fw0 != ms.fw) {
-            const float4 gw = wtab ? wtab[I.fw0] : __ldg(reinterpret_cast<const float4 *>(gwt) + I.fw0);
-            build_rows<DT>(ms.M, ws.m, subgrids, base, I.key0, gw, g, vec_ok, lane, j);
-            ms.key = I.key0;
-            ms.fw = I.fw0;
-        }
+    const float4 gw = w_row(A, fw);
+    const int64_t col = base + key + (int64_t)(A.lane & 7) * g.nz + (int64_t)(A.lane >> 3) * g.row_stride;
+    const bool vec = vec_footprint<DT>(A.vec_ok, key);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int r = 8 * (k ^ j) + p;
-            P[k] = quarter_sum(ms.M, S, r, j);
+    for (int k = 0; k < 2; ++k)
+        m[k] = footprint_point<DT>(A.subgrids, col + (int64_t)(4 * k) * g.row_stride, gw, vec);
+}
+
+__device__ __forceinline__ void store_points(MSlot &slot, const float2 (&m)[2], int lane)
+{
+    (&slot.m[0][0])[lane] = m[0];
+    (&slot.m[4][0])[lane] = m[1];
+}
+
+// The two visibilities of a lane in a step.
+struct Vis2 {
+    int key[2];         // footprint start, -1: invalid or past the end of the step
+    int fw[2];          // w row
+    int ru[2], rv[2];   // g_u and g_v rows
+};
+
+__device__ __forceinline__ Vis2 snap_step(const Step &b, const Coords3 (&c)[2], const Geometry &g,
+                                          DeviceStatus *status, int lane)
+{
+    Vis2 r;
+    bool bad[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const bool in = lane + kBatch * h < b.n;
+        VisCoords vc;
+        bool valid = in && visibility_coords(c[h].u, c[h].v, c[h].w, g, vc);
+#ifdef DEGRID_BOUNDS_CHECK
+        if (valid)
+            valid = indices_in_bounds((vc.y0 * g.nx + vc.x0) * g.nz + vc.z0, vc.fu, vc.fv, vc.fw, g, status);
+#endif
+        r.key[h] = valid ? (vc.y0 * g.nx + vc.x0) * g.nz + vc.z0 : -1;
+        r.fw[h] = valid ? vc.fw : 0;
+        r.ru[h] = valid ? vc.fu : 0;
+        r.rv[h] = valid ? vc.fv : 0;
+        bad[h] = in && !valid;
+    }
+    if (__any_sync(kFull, bad[0] || bad[1])) {
+        const int n = __popc(__ballot_sync(kFull, bad[0])) + __popc(__ballot_sync(kFull, bad[1]));
+        if (lane == 0)
+            atomicAdd(&status->n_invalid, (unsigned long long)n);
+    }
+    return r;
+}
+
+// A table row in registers.
+struct Row8 {
+    float w[kUV];
+};
+
+// Starts the copies of the step's g_u and g_v rows (two lanes per 32-byte
+// row, so each row is one request; one cp.async group).
+__device__ __forceinline__ void copy_rows(RowStage (&st)[2], const Vis2 &s, const float *__restrict__ guv, int lane)
+{
+    const int half = lane & 1;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const int row = (lane >> 1) + 16 * m;
+            const int xu = __shfl_sync(kFull, s.ru[h], row);
+            const int xv = __shfl_sync(kFull, s.rv[h], row);
+            cp_async16(smem_u32(&st[h].u[row][RowStage::slot(row, half)]), guv + (size_t)xu * kUVRow + 4 * half);
+            cp_async16(smem_u32(&st[h].v[row][RowStage::slot(row, half)]), guv + (size_t)xv * kUVRow + 4 * half);
         }
-    } else if (DIRECT && I.runs >= direct_runs) {
-        // Short runs: every visibility is summed from its own footprint
-        // (pass k covers visibilities 8k .. 8k + 7; invalid ones stay zero).
-        // Pays off when the footprints of a half overlap (slowly moving
-        // lists whose w row changes often: the other visibilities keep them
-        // in L1); for footprints scattered over the subgrid the cooperative
-        // M builds below read it in longer contiguous pieces and win.  A
-        // separate kernel instance, so the register budget of the plain
-        // path is untouched.
-#pragma unroll 1
-        for (int k = 0; k < 4; ++k) {
-            const int r = 8 * k + p;
-            const int kr = __shfl_sync(kFull, I.key, r);
-            const int fr = __shfl_sync(kFull, I.fw, r);
-            float2 acc = make_float2(0.f, 0.f);
-            if (kr >= 0) {
-                const float4 gw = wtab ? wtab[fr] : __ldg(reinterpret_cast<const float4 *>(gwt) + fr);
-                acc = quarter_sum_direct<DT>(subgrids, base, kr, gw, S, r, j, g, vec_ok);
+    cp_async_commit();
+}
+
+__device__ __forceinline__ Row8 stage_row(const float4 (&row)[2], int lane)
+{
+    const float4 a = row[RowStage::slot(lane, 0)], b = row[RowStage::slot(lane, 1)];
+    return Row8{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
+}
+
+// sum_a g[a] m[a] over one row of M (4 float4 in shared memory), as packed
+// pairs (re, im) * (g, g): one FFMA2 per product, each half rounded exactly
+// as a scalar FMA.
+__device__ __forceinline__ float2 row_sum(const float4 (&m)[4], const Row8 &g)
+{
+    float2 t = __fmul2_rn(make_float2(m[0].x, m[0].y), make_float2(g.w[0], g.w[0]));
+    t = __ffma2_rn(make_float2(m[0].z, m[0].w), make_float2(g.w[1], g.w[1]), t);
+#pragma unroll
+    for (int a = 1; a < 4; ++a) {
+        t = __ffma2_rn(make_float2(m[a].x, m[a].y), make_float2(g.w[2 * a], g.w[2 * a]), t);
+        t = __ffma2_rn(make_float2(m[a].z, m[a].w), make_float2(g.w[2 * a + 1], g.w[2 * a + 1]), t);
+    }
+    return t;
+}
+
+__device__ __forceinline__ void read_row(float4 (&m)[4], const MSlot &slot, int b)
+{
+    const float4 *p = reinterpret_cast<const float4 *>(&slot.m[b][0]);
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+        m[a] = p[a];
+}
+
+// (Q0 + Q2) + (Q1 + Q3), the order every kernel of the library uses; the
+// compensated form makes the three additions error-free, sums their errors
+// and adds them back once.
+template <bool COMP>
+__device__ __forceinline__ float combine(float q0, float q1, float q2, float q3)
+{
+    if (!COMP)
+        return (q0 + q2) + (q1 + q3);
+    float e0, e1, e;
+    const float s0 = two_sum(q0, q2, e0), s1 = two_sum(q1, q3, e1);
+    const float v = two_sum(s0, s1, e);
+    return v + (e + (e0 + e1));
+}
+
+// The lane's two visibilities from the footprints in s0 and s1 (with SHARED
+// the same slot for both: read once) and their rows in the stage.  Quarter j
+// is rows 2j and 2j + 1, g_v[2j + 1] R_{2j + 1} + g_v[2j] R_{2j} with
+// R_b = sum_a g_u[a] M[b][a].
+template <bool COMP, bool SHARED>
+__device__ __forceinline__ void sum_step(float2 (&V)[2], const MSlot &s0, const MSlot &s1, const RowStage (&st)[2],
+                                         int lane)
+{
+    float2 Q[2][4];
+    const Row8 gu[2] = {stage_row(st[0].u[lane], lane), stage_row(st[1].u[lane], lane)};
+#pragma unroll
+    for (int jj = 0; jj < 2; ++jj) {
+        const float4 gv[2] = {st[0].v[lane][RowStage::slot(lane, jj)], st[1].v[lane][RowStage::slot(lane, jj)]};
+#pragma unroll
+        for (int j2 = 0; j2 < 2; ++j2) {
+            const int j = 2 * jj + j2;
+            float2 R[2][2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int b = 2 * j + i;
+                float4 m[4];
+                read_row(m, s0, b);
+                R[0][i] = row_sum(m, gu[0]);
+                if (!SHARED)
+                    read_row(m, s1, b);
+                R[1][i] = row_sum(m, gu[1]);
             }
-            ws.part[k][lane] = acc;
-        }
-        __syncwarp();
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            P[k] = ws.part[k ^ j][lane];
-        __syncwarp();
-    } else {
-        // Pass k covers visibilities 8k .. 8k + 7 here, so a change of
-        // footprint inside a run of the list touches one pass.  Each pass is
-        // summed once per distinct (footprint, w row) among its visibilities,
-        // every lane keeping the sum that matches its own (invalid ones, key
-        // -1, stay zero); the partials then move to the slots of the permuted
-        // order, slot k = pass k ^ j.
-#pragma unroll 1
-        for (int k = 0; k < 4; ++k) {
-            const int r = 8 * k + p;
-            const int kr = __shfl_sync(kFull, I.key, r);
-            const int fr = __shfl_sync(kFull, I.fw, r);
-            bool done = kr < 0;
-            float2 acc = make_float2(0.f, 0.f);
-#pragma unroll 1
-            while (true) {
-                const unsigned todo = __ballot_sync(kFull, !done);
-                if (todo == 0)
-                    break;
-                const int leader = __ffs(todo) - 1;
-                const int lk = __shfl_sync(kFull, kr, leader);
-                const int lf = __shfl_sync(kFull, fr, leader);
-                if (lk != ms.key || lf != ms.fw) {
-                    const float4 gw = wtab ? wtab[lf] : __ldg(reinterpret_cast<const float4 *>(gwt) + lf);
-                    build_rows<DT>(ms.M, ws.m, subgrids, base, lk, gw, g, vec_ok, lane, j);
-                    ms.key = lk;
-                    ms.fw = lf;
-                }
-                const float2 x = quarter_sum(ms.M, S, r, j);
-                const bool mine = !done && kr == lk && fr == lf;
-                if (mine)
-                    acc = x;
-                done = done || mine;
+            for (int h = 0; h < 2; ++h) {
+                const float ve = j2 ? gv[h].z : gv[h].x, vo = j2 ? gv[h].w : gv[h].y;
+                Q[h][j] = __ffma2_rn(R[h][1], make_float2(vo, vo), __fmul2_rn(R[h][0], make_float2(ve, ve)));
             }
-            ws.part[k][lane] = acc;
         }
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            P[k] = ws.part[k ^ j][lane];
-        __syncwarp();
     }
-    reduce_store<DT, COMP>(P, h, sc, vis_out, lane);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        V[h].x = combine<COMP>(Q[h][0].x, Q[h][1].x, Q[h][2].x, Q[h][3].x);
+        V[h].y = combine<COMP>(Q[h][0].y, Q[h][1].y, Q[h][2].y, Q[h][3].y);
+    }
 }
 
-// Both halves of a full step share one footprint and w row (the common
-// case on dense lists): their eight passes are summed in one block, so the
-// scheduler can interleave the two halves' loads and FMA chains.
+// The most recently built footprint of a warp: (key, fw) of the current
+// subgrid is in slot `slot` (key -2: none).
+struct MCache {
+    int key, fw, slot;
+};
+
+// A step that does not continue the cached run alone: its runs (maximal
+// sequences of equal footprint and w row in list order) are built up to
+// kSlots at a time, two footprints' loads in flight together, and each round
+// is summed once, every lane reading the slots of its own visibilities' runs.
 template <int DT, bool COMP>
-__device__ __forceinline__ void sum_step_uniform(MState &ms, WarpSmem &ws, const RowStage &S0,
-                                                 const RowStage &S1, const Issued &I0, const Issued &I1,
-                                                 const Batch &b, const void *__restrict__ subgrids,
-                                                 int64_t base, float sc, const Geometry &g,
-                                                 const float4 *wtab, const float *__restrict__ gwt,
-                                                 float2 *__restrict__ vis_out, bool vec_ok,
-                                                 int lane, int p, int j)
+__device__ __forceinline__ void sum_runs(float2 (&V)[2], MCache &mc, WarpSmem &ws, const RowStage (&st)[2],
+                                         int64_t base, const Vis2 &vis,
+                                         const Geometry &g, const BuildArgs &A)
 {
-    if (I0.key0 != ms.key || I0.fw0 != ms.fw) {
-        const float4 gw = wtab ? wtab[I0.fw0] : __ldg(reinterpret_cast<const float4 *>(gwt) + I0.fw0);
-        build_rows<DT>(ms.M, ws.m, subgrids, base, I0.key0, gw, g, vec_ok, lane, j);
-        ms.key = I0.key0;
-        ms.fw = I0.fw0;
+    const int lane = A.lane;
+    __syncwarp();                       // earlier steps' reads of the slots are done
+    unsigned heads[2];
+    int run[2];                         // run of the lane's visibilities
+    {
+        int kp = __shfl_up_sync(kFull, vis.key[0], 1), fp = __shfl_up_sync(kFull, vis.fw[0], 1);
+        heads[0] = __ballot_sync(kFull, vis.key[0] >= 0 && (lane == 0 || vis.key[0] != kp || vis.fw[0] != fp));
+        // visibility 32 follows visibility 31
+        kp = __shfl_sync(kFull, lane == 31 ? vis.key[0] : vis.key[1], (lane + 31) & 31);
+        fp = __shfl_sync(kFull, lane == 31 ? vis.fw[0] : vis.fw[1], (lane + 31) & 31);
+        heads[1] = __ballot_sync(kFull, vis.key[1] >= 0 && (vis.key[1] != kp || vis.fw[1] != fp));
+        const unsigned upto = 0xffffffffu >> (31 - lane);
+        run[0] = __popc(heads[0] & upto) - 1;
+        run[1] = __popc(heads[0]) + __popc(heads[1] & upto) - 1;
     }
-    float2 P0[4], P1[4];
+    const int n_runs = __popc(heads[0]) + __popc(heads[1]);
+    V[0] = V[1] = make_float2(0.f, 0.f);
+    for (int first = 0; first < n_runs; first += kSlots) {
+        const int n = min(kSlots, n_runs - first);
+        int todo = n;
+        const auto head = [&](int &key, int &fw) {          // takes the next run's head off the list
+            const int h = heads[0] ? 0 : 1;
+            const int src = __ffs(h ? heads[1] : heads[0]) - 1;
+            key = __shfl_sync(kFull, h ? vis.key[1] : vis.key[0], src);
+            fw = __shfl_sync(kFull, h ? vis.fw[1] : vis.fw[0], src);
+            if (h)
+                heads[1] &= heads[1] - 1;
+            else
+                heads[0] &= heads[0] - 1;
+        };
+        int key, fw;
+        head(key, fw);
+        bool have = true;               // (key, fw) is a run that is not built yet
+        if (key == mc.key && fw == mc.fw) {
+            --todo;                     // the first run continues the cached one
+            have = false;
+        }
+        const int start = (mc.slot + (have ? 1 : 0)) & (kSlots - 1);
+        // builds the next N runs, their loads in flight together
+        const auto build = [&](auto n_runs_built) {
+            constexpr int N = decltype(n_runs_built)::value;
+            int k[N], f[N];
+            float2 m[N][2];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int r = 8 * (k ^ j) + p;
-        P0[k] = quarter_sum(ms.M, S0, r, j);
-        P1[k] = quarter_sum(ms.M, S1, r, j);
+            for (int i = 0; i < N; ++i) {
+                if (!have)
+                    head(key, fw);
+                have = false;
+                k[i] = key;
+                f[i] = fw;
+            }
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+                build_points<DT>(m[i], base, k[i], f[i], g, A);
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                mc.slot = (mc.slot + 1) & (kSlots - 1);
+                store_points(ws.slot[mc.slot], m[i], lane);
+            }
+            mc.key = key;
+            mc.fw = fw;
+            todo -= N;
+        };
+        while (todo >= 2)               // (four at a time cost registers: lines 225 us instead of 211)
+            build(std::integral_constant<int, 2>{});
+        if (todo >= 1)
+            build(std::integral_constant<int, 1>{});
+        __syncwarp();
+        const bool mine0 = vis.key[0] >= 0 && run[0] >= first && run[0] < first + n;
+        const bool mine1 = vis.key[1] >= 0 && run[1] >= first && run[1] < first + n;
+        float2 x[2];
+        sum_step<COMP, false>(x, ws.slot[(start + (mine0 ? run[0] - first : 0)) & (kSlots - 1)],
+                              ws.slot[(start + (mine1 ? run[1] - first : 0)) & (kSlots - 1)], st, lane);
+        if (mine0)
+            V[0] = x[0];
+        if (mine1)
+            V[1] = x[1];
+        __syncwarp();                   // slots read before the next round builds into them
     }
-    reduce_store<DT, COMP>(P0, half_of(b, 0), sc, vis_out, lane);
-    reduce_store<DT, COMP>(P1, half_of(b, 1), sc, vis_out, lane);
 }
 
-template <int DT, bool COMP, bool DIRECT>
-__global__ void __launch_bounds__(kMaxWarps * kWarp, DG_DEGRID_MIN_BLOCKS)
+template <int DT, bool COMP>
+__global__ void __launch_bounds__(kMaxWarps * kWarp, 2)
 degrid_kernel(const Geometry g, const void *__restrict__ subgrids, const float *__restrict__ scale,
               const double *__restrict__ uvw, const float *__restrict__ guv,
               const float *__restrict__ gwt, const Schedule sched, float2 *__restrict__ vis_out,
-              DeviceStatus *__restrict__ status, const int direct_runs, const bool vec_ok,
-              const bool prefetch_uvw)
+              DeviceStatus *__restrict__ status, const bool vec_ok, const bool prefetch_uvw)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     // [w table (optional)] [one WarpSmem per warp]
     WarpSmem &ws = reinterpret_cast<WarpSmem *>(smem_raw + wtable_bytes(g))[threadIdx.x >> 5];
     const float4 *wtab = load_wtable(g, gwt, smem_raw);
     const int lane = threadIdx.x & 31;
-    const int p = lane & 7, j = lane >> 3;
+    const BuildArgs A{subgrids, wtab, gwt, vec_ok, lane};
 
     // coordinates in device memory are prefetched into L2 a chunk ahead;
     // coordinates read in place from host memory are not (the host link
     // bounds those calls, and one batch of lead hides its latency)
     pdl_wait();                         // the chunk table is complete
-    ClaimerT<kBatchVis> claimer(sched, lane,
-                                Prefetch{prefetch_uvw ? uvw : nullptr, 3 * (int)sizeof(double), nullptr, 0});
-    Batch bB = claimer.claim();         // rows in flight
-    if (bB.n == 0)
+    Steps steps{ClaimerT<kStepVis>(sched, lane, Prefetch{prefetch_uvw ? uvw : nullptr, 3 * (int)sizeof(double),
+                                                         nullptr, 0}),
+                uvw + 3 * lane, vis_out + lane};
+    Step pA = steps.claim();            // the step being summed
+    if (pA.n == 0)
         return;
-    Issued iB0 = issue_rows<RowStage>(half_of(bB, 0), load_uvw(uvw, half_of(bB, 0), lane), g,
-                                            ws.st[0][0], guv, lane, status, false);
-    Issued iB1 = issue_rows<RowStage>(half_of(bB, 1), load_uvw(uvw, half_of(bB, 1), lane), g,
-                                            ws.st[0][1], guv, lane, status, true);
-    Batch bC = claimer.advance(bB);     // coordinates in registers
-    Coords3 cC0 = load_uvw(uvw, half_of(bC, 0), lane);
-    Coords3 cC1 = load_uvw(uvw, half_of(bC, 1), lane);
+    Coords3 c[2];
+    load_coords(c, pA, lane);
+    Vis2 vA = snap_step(pA, c, g, status, lane);
+    copy_rows(ws.st, vA, guv, lane);
+    Step pB = steps.advance(pA);        // the step after it, its coordinates in registers
+    load_coords(c, pB, lane);
 
-    int stage = 0;
-    MState ms;
-    ms.key = -2;
-    ms.fw = -1;
+    MCache mc{-2, -1, 0};
     int m_s = -1;
     int64_t base = 0;
     float sc = 1.f;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int a = 0; a < 8; ++a)
-            ms.M[i][a] = make_float2(0.f, 0.f);
+    while (true) {
+        const Vis2 vB = snap_step(pB, c, g, status, lane);
+        const Step pC = steps.advance(pB);
+        load_coords(c, pC, lane);
 
-    while (bB.n > 0) {
-        const Batch bA = bB;            // summed in this iteration
-        const Issued iA0 = iB0, iA1 = iB1;
-        const int sA = stage;
-        bB = bC;
-        if (bB.n > 0) {
-            iB0 = issue_rows<RowStage>(half_of(bB, 0), cC0, g, ws.st[sA ^ 1][0], guv, lane, status,
-                                             false);
-            iB1 = issue_rows<RowStage>(half_of(bB, 1), cC1, g, ws.st[sA ^ 1][1], guv, lane, status,
-                                             true);
-        }
-        bC = claimer.advance(bC);
-        cC0 = load_uvw(uvw, half_of(bC, 0), lane);
-        cC1 = load_uvw(uvw, half_of(bC, 1), lane);
-        if (bB.n > 0)
-            cp_async_wait<1>();         // the stage of batch A; batch B may stay in flight
-        else
-            cp_async_wait<0>();
-        __syncwarp();
-
-        if (bA.s != m_s) {
-            m_s = bA.s;
-            ms.key = -2;
-            base = (int64_t)bA.s * g.plane;
+        if (pA.s != m_s) {
+            m_s = pA.s;
+            mc.key = -2;
+            base = (int64_t)pA.s * g.plane;
             if (DT != DG_C64)
-                sc = __ldg(scale + bA.s);
+                sc = __ldg(scale + pA.s);
         }
-        if (iA0.uniform && iA1.uniform && iA0.key0 == iA1.key0 && iA0.fw0 == iA1.fw0 &&
-            bA.n == kBatchVis) {
-            sum_step_uniform<DT, COMP>(ms, ws, ws.st[sA][0], ws.st[sA][1], iA0, iA1, bA, subgrids,
-                                            base, sc, g, wtab, gwt, vis_out, vec_ok, lane, p, j);
-        } else {
-            sum_half<DT, COMP, DIRECT>(ms, ws, ws.st[sA][0], iA0, half_of(bA, 0), subgrids, base, sc,
-                                            g, wtab, gwt, vis_out, direct_runs, vec_ok, lane, p, j);
-            if (bA.n > kBatch)
-                sum_half<DT, COMP, DIRECT>(ms, ws, ws.st[sA][1], iA1, half_of(bA, 1), subgrids, base,
-                                                sc, g, wtab, gwt, vis_out, direct_runs, vec_ok, lane, p,
-                                                j);
+        cp_async_wait<0>();
+        __syncwarp();                   // every lane's copies
+        float2 V[2];
+        if (__all_sync(kFull, vA.key[0] == mc.key && vA.fw[0] == mc.fw && vA.key[1] == mc.key && vA.fw[1] == mc.fw))
+            // the whole step continues the cached run (nearly always, on dense lists)
+            sum_step<COMP, true>(V, ws.slot[mc.slot], ws.slot[mc.slot], ws.st, lane);
+        else
+            sum_runs<DT, COMP>(V, mc, ws, ws.st, base, vA, g, A);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (DT != DG_C64)
+                V[h] = __fmul2_rn(V[h], make_float2(sc, sc));
+            if (lane + kBatch * h < pA.n)
+                pA.out[kBatch * h] = V[h];
         }
-        __syncwarp();
-        stage ^= 1;
+        if (pB.n == 0)
+            break;
+        __syncwarp();                   // the rows have been read
+        copy_rows(ws.st, vB, guv, lane);
+        vA = vB;
+        pA = pB;
+        pB = pC;
     }
+    cp_async_wait<0>();
 }
 
 size_t smem_bytes(const degrid_plan *p, int warps)
@@ -397,20 +466,20 @@ size_t smem_bytes(const degrid_plan *p, int warps)
 }
 
 // Dynamic shared memory opened so far for a kernel instance on a device.
-template <int DT, bool COMP, bool DIRECT>
+template <int DT, bool COMP>
 std::atomic<size_t> &smem_record(int device)
 {
     static std::atomic<size_t> table[kMaxDevices];
     return dg_smem_record(table, device);
 }
 
-template <int DT, bool COMP, bool DIRECT>
+template <int DT, bool COMP>
 cudaError_t launch(degrid_plan *p, cudaStream_t st, const void *subgrids, const float *scale,
                    const double *uvw, float2 *out, const Schedule &sched, int grid_blocks)
 {
     const int threads = p->warps_per_block * kWarp;
     const size_t smem = smem_bytes(p, p->warps_per_block);
-    cudaError_t e = dg_open_smem(smem_record<DT, COMP, DIRECT>(p->device), degrid_kernel<DT, COMP, DIRECT>,
+    cudaError_t e = dg_open_smem(smem_record<DT, COMP>(p->device), degrid_kernel<DT, COMP>,
                                  smem);
     if (e != cudaSuccess)
         return e;
@@ -418,55 +487,40 @@ cudaError_t launch(degrid_plan *p, cudaStream_t st, const void *subgrids, const 
     // elements per 16 bytes
     const bool vec_ok = (reinterpret_cast<uintptr_t>(subgrids) & 15) == 0 &&
                         p->geo.nz % Storage<DT>::kQuad == 0;
-    return launch_pdl(degrid_kernel<DT, COMP, DIRECT>, dim3(grid_blocks), dim3(threads), smem, st,
+    return launch_pdl(degrid_kernel<DT, COMP>, dim3(grid_blocks), dim3(threads), smem, st,
                       p->geo, subgrids, scale, uvw, (const float *)p->guv, (const float *)p->gw, sched, out,
-                      p->status, p->direct_runs, vec_ok, !p->host_inputs);
+                      p->status, vec_ok, !p->host_inputs);
 }
 
-template <int DT, bool COMP, bool DIRECT>
+template <int DT, bool COMP>
 int max_blocks(degrid_plan *p)
 {
     int n = 0;
     const size_t smem = smem_bytes(p, p->warps_per_block);
-    if (dg_open_smem(smem_record<DT, COMP, DIRECT>(p->device), degrid_kernel<DT, COMP, DIRECT>, smem) !=
+    if (dg_open_smem(smem_record<DT, COMP>(p->device), degrid_kernel<DT, COMP>, smem) !=
         cudaSuccess)
         return 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, degrid_kernel<DT, COMP, DIRECT>,
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, degrid_kernel<DT, COMP>,
                                                       p->warps_per_block * kWarp, smem) != cudaSuccess)
         return 1;
     return n > 0 ? n : 1;
 }
 
-// Kernel instance of a plan: storage type, compensated reduction, and one of
-// two summing forms (footprint cache; with the direct arm).  Plans with a 2D
-// G_uv table have their own kernel (table2d.cu).
-template <int DT, bool COMP>
-cudaError_t launch_form(degrid_plan *p, cudaStream_t st, const void *subgrids, const float *scale,
-                        const double *uvw, float2 *out, const Schedule &sched, int grid_blocks)
-{
-    if (p->direct_runs < DG_DIRECT_RUNS_NEVER)
-        return launch<DT, COMP, true>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
-    return launch<DT, COMP, false>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
-}
-
-template <int DT, bool COMP>
-int max_blocks_form(degrid_plan *p)
-{
-    return p->direct_runs < DG_DIRECT_RUNS_NEVER ? max_blocks<DT, COMP, true>(p) : max_blocks<DT, COMP, false>(p);
-}
-
+// Kernel instance of a plan: storage type and compensated reduction.  Plans
+// with a 2D G_uv table (table2d.cu) or with the direct arm (direct.cu) have
+// kernels of their own.
 template <int DT>
 cudaError_t launch_dt(degrid_plan *p, cudaStream_t st, const void *subgrids, const float *scale,
                       const double *uvw, float2 *out, const Schedule &sched, int grid_blocks)
 {
-    return p->compensated ? launch_form<DT, true>(p, st, subgrids, scale, uvw, out, sched, grid_blocks)
-                          : launch_form<DT, false>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
+    return p->compensated ? launch<DT, true>(p, st, subgrids, scale, uvw, out, sched, grid_blocks)
+                          : launch<DT, false>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
 }
 
 template <int DT>
 int max_blocks_dt(degrid_plan *p)
 {
-    return p->compensated ? max_blocks_form<DT, true>(p) : max_blocks_form<DT, false>(p);
+    return p->compensated ? max_blocks<DT, true>(p) : max_blocks<DT, false>(p);
 }
 
 }  // namespace
@@ -480,6 +534,8 @@ cudaError_t dg_launch_degrid(degrid_plan *p, cudaStream_t st, const void *subgri
     (void)vis_offsets;
     if (p->guv2)
         return dg_launch_degrid_2d(p, st, subgrids, scale, uvw, out_f, grid_blocks);
+    if (p->direct_runs < DG_DIRECT_RUNS_NEVER)
+        return dg_launch_degrid_direct(p, st, subgrids, scale, uvw, out_f, grid_blocks);
     Schedule sched{p->chunks, p->n_chunks, p->work_counter};
     float2 *out = reinterpret_cast<float2 *>(out_f);
     switch (p->dtype) {
@@ -498,6 +554,8 @@ int dg_max_blocks_per_sm_degrid(degrid_plan *p)
     using namespace dg;
     if (p->guv2)
         return dg_max_blocks_per_sm_degrid_2d(p);
+    if (p->direct_runs < DG_DIRECT_RUNS_NEVER)
+        return dg_max_blocks_per_sm_degrid_direct(p);
     switch (p->dtype) {
     case DG_C64: return max_blocks_dt<DG_C64>(p);
     case DG_C32_F16: return max_blocks_dt<DG_C32_F16>(p);

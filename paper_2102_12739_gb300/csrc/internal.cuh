@@ -248,7 +248,7 @@ struct degrid_plan {
     int warps_per_block;
     int blocks_per_sm;
     int compensated;            // compensated (TwoSum) reduction of the lane partials
-    int direct_runs;            // non-uniform halves with at least this many runs take the direct sum
+    int direct_runs;            // below DG_DIRECT_RUNS_NEVER: the direct kernel, halves with at least this many runs summed directly
     int gather;                 // sum through the gather kernel (gather.cu)
     int host_direct;            // degrid_execute_host reads page-locked host inputs in place
     int host_inputs;            // set during such a call: the kernel's inputs are in host memory
@@ -358,9 +358,12 @@ cudaError_t dg_launch_scatter(degrid_plan *p, cudaStream_t st, int n_subgrids, c
 int dg_scatter_warps();                         // warps per CTA of the scattered gridding kernel
 bool dg_gather_supported(const degrid_plan *p);
 int dg_max_blocks_per_sm_degrid(degrid_plan *p);
-// plans with a 2D G_uv table (called through the two above)
+// plans with a 2D G_uv table, and with the direct arm (called through the two above)
 cudaError_t dg_launch_degrid_2d(degrid_plan *p, cudaStream_t st, const void *subgrids, const float *scale,
                                 const double *uvw, float *vis_out, int grid_blocks);
 int dg_max_blocks_per_sm_degrid_2d(degrid_plan *p);
+cudaError_t dg_launch_degrid_direct(degrid_plan *p, cudaStream_t st, const void *subgrids, const float *scale,
+                                    const double *uvw, float *vis_out, int grid_blocks);
+int dg_max_blocks_per_sm_degrid_direct(degrid_plan *p);
 int dg_max_warps_per_block();        // largest warps_per_block the kernels are built for
 int dg_max_blocks_per_sm_adjoint(degrid_plan *p);

@@ -1139,3 +1139,46 @@ def test_table2d_steps_of_many_runs(dtype, comp, nz):
         assert p.status() == bad == 5
     assert np.linalg.norm(got - ref) <= 2e-6 * np.linalg.norm(ref)
     assert np.all(got[[5, 70, 71, 133, 200]] == 0)
+
+
+@pytest.mark.parametrize("dtype,comp", [("c64", False), ("f16", True), ("bf16", False)])
+@pytest.mark.parametrize("nz", [4, 6])
+def test_steps_of_many_runs(dtype, comp, nz):
+    # steps of 64 with 1, 2, 8, 9, 17, 33 and 64 runs of equal footprint and
+    # w row (a warp holds 8 footprints), a run over the middle of a step, runs
+    # that continue into the next step, invalid visibilities inside runs, a
+    # subgrid change and ragged ends; against the oracle and, bit for bit, the
+    # direct arm
+    d = dev()
+    shape = (40, 48, nz)
+    rng = np.random.default_rng(nz)
+    steps = []
+    for n_runs in (1, 1, 2, 8, 9, 17, 33, 64, 1, 3):
+        p = np.stack([rng.uniform(4, 40, n_runs), rng.uniform(4, 32, n_runs), rng.uniform(1.0, nz - 2.01, n_runs)], 1)
+        at = np.sort(rng.integers(0, n_runs, 64)) if n_runs < 64 else np.arange(64)
+        steps.append(p[at] + np.array([1e-6, 1e-6, 0.0]) * np.arange(64)[:, None])
+    uvw = np.concatenate(steps + [steps[0][:41], steps[3][:64], steps[2][:7]])
+    bad = [5, 70, 71, 133, 200, 300]
+    uvw[bad] = [[np.nan, 9, 1.5], [1e9, 9, 1.5], [-3, 9, 1.5], [9, 1e300, 1.5], [9, 9, 77.0], [9, -1e-300, 1.5]]
+    offs = np.array([0, 681, 681, len(uvw)])
+    sub = torch.from_numpy(synth.subgrid_stack(3, shape=shape)).to(d)
+    codes, scale = (sub, None) if dtype == "c64" else dg.pack_subgrids(sub, dtype)
+    stored = sub.cpu().numpy().astype(np.complex128)
+    if dtype != "c64":
+        q = codes.float().cpu().numpy().astype(np.float64) * scale.cpu().numpy().astype(np.float64)[:, None, None, None, None]
+        stored = q[..., 0] + 1j * q[..., 1]
+    ref, n_bad = oracle.degrid(G_UV, G_W, stored, uvw, offs)
+    assert n_bad == len(bad)
+    outs = []
+    with dg.DegridPlan(shape=shape, dtype=dtype, device=d, compensated=comp) as p:
+        for direct in (dg._native.DG_DIRECT_RUNS_NEVER, 1):
+            for chunk in (64, 256, 1024):
+                p.set_direct_runs(direct)
+                p.set_tuning(chunk, 8, 0)
+                outs.append(p.degrid(codes, torch.from_numpy(uvw).to(d), torch.from_numpy(offs).to(d),
+                                     scale=scale).cpu().numpy())
+                assert p.status() == len(bad)
+    assert rel_l2(outs[0], ref) <= 2e-6
+    assert np.all(outs[0][bad] == 0)
+    for o in outs[1:]:
+        np.testing.assert_array_equal(o.view(np.uint64), outs[0].view(np.uint64))
