@@ -19,6 +19,7 @@ Main objects:
 from __future__ import annotations
 
 import ctypes
+import functools
 from typing import Optional
 
 import numpy as np
@@ -34,25 +35,33 @@ __all__ = ["DegridPlan", "DegridFn", "DegridError", "pack_subgrids", "degrid", "
 DTYPES = {"c64": DG_C64, "f16": DG_C32_F16, "bf16": DG_C32_BF16}
 
 
+@functools.lru_cache(maxsize=None)
 def _torch():
     import torch
     return torch
 
 
-def _vp(t) -> Optional[ctypes.c_void_p]:
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+def _vp(t) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
-def _stream_handle(stream, device):
-    torch = _torch()
+def _stream_handle(stream, device) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream(device)
-    return ctypes.c_void_p(stream.cuda_stream)
+        return _raw_stream()(device.index)
+    return stream.cuda_stream
+
+
+@functools.lru_cache(maxsize=None)
+def _raw_stream():
+    """Device index -> handle of PyTorch's current stream there, without the
+    stream object where PyTorch offers it (2 us of a 19 us call)."""
+    torch = _torch()
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw if raw is not None else lambda index: torch.cuda.current_stream(index).cuda_stream
 
 
 def _need(t, name, dtype, device, shape=None):
-    torch = _torch()
-    if not isinstance(t, torch.Tensor):
+    if not isinstance(t, _torch().Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.dtype != dtype:
         raise TypeError(f"{name} must have dtype {dtype}, got {t.dtype}")
@@ -60,7 +69,7 @@ def _need(t, name, dtype, device, shape=None):
         raise ValueError(f"{name} must live on {device}, got {t.device}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
 
 

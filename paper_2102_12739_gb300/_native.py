@@ -99,6 +99,9 @@ def lib_path() -> str:
 def load(build_if_missing: bool = True):
     """Load libdegrid.so (building it first if needed) and bind signatures."""
     global _lib
+    lib = _lib
+    if lib is not None:                 # every compute call comes through here
+        return lib
     with _lock:
         if _lib is None:
             variant = _variant()

@@ -16,13 +16,17 @@ cudaError_t dg_launch_pack(cudaStream_t st, dg_dtype dtype, int n_subgrids, int6
 namespace {
 
 // Makes `device` current for the duration of an API call and restores the
-// caller's device afterwards.
+// caller's device afterwards (nothing to set or restore if it is current).
 struct DeviceGuard {
     int prev = -1;
     bool ok = false;
     explicit DeviceGuard(int device)
     {
-        ok = cudaGetDevice(&prev) == cudaSuccess && cudaSetDevice(device) == cudaSuccess;
+        ok = cudaGetDevice(&prev) == cudaSuccess;
+        if (ok && prev == device)
+            prev = -1;
+        else if (ok)
+            ok = cudaSetDevice(device) == cudaSuccess;
     }
     ~DeviceGuard()
     {
