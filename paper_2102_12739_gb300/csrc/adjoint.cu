@@ -217,12 +217,13 @@ __device__ __forceinline__ void accumulate_half(RunState &rs, WarpSmem &ws, cons
     }
 }
 
-template <bool T2D, bool kVec4>
+// SMALL: by pieces, without a chunk table.
+template <bool T2D, bool kVec4, bool SMALL>
 __global__ void __launch_bounds__(kMaxWarps * kWarp, DG_ADJOINT_MIN_BLOCKS)
 adjoint_kernel(const Geometry g, const double *__restrict__ uvw, const float2 *__restrict__ vis_in,
                const float *__restrict__ guv, const float *__restrict__ gwt, const Schedule sched,
                float2 *__restrict__ sub_out, DeviceStatus *__restrict__ status,
-               const float *__restrict__ g2)
+               const float *__restrict__ g2, const Pieces pieces)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     WarpSmem &ws = reinterpret_cast<WarpSmem *>(smem_raw + wtable_bytes(g))[threadIdx.x >> 5];
@@ -231,13 +232,24 @@ adjoint_kernel(const Geometry g, const double *__restrict__ uvw, const float2 *_
     const int p = lane & 7, j = lane >> 3;
 
     pdl_wait();                         // the chunk table (and the zeroed output) are complete
-    ClaimerT<kStepVis> claimer(sched, lane, Prefetch{uvw, 3 * (int)sizeof(double), vis_in, (int)sizeof(float2)});
+    const auto make_claimer = [&] {
+        if constexpr (SMALL)
+            return PieceClaimerT<kStepVis>(pieces, lane);
+        else
+            return ClaimerT<kStepVis>(sched, lane,
+                                      Prefetch{uvw, 3 * (int)sizeof(double), vis_in, (int)sizeof(float2)});
+    };
+    auto claimer = make_claimer();
+    const bool checks = SMALL && blockIdx.x == 0 && threadIdx.x < kWarp;
     Batch bB = claimer.claim();
-    if (bB.n == 0)
+    if (bB.n == 0) {
+        if (checks)
+            check_offsets(pieces, status, lane);
         return;
-    Issued iB0 = issue_rows<RowStage, !T2D>(half_of(bB, 0), load_uvw(uvw, half_of(bB, 0), lane), g,
+    }
+    Issued iB0 = issue_rows<RowStage, !T2D, SMALL>(half_of(bB, 0), load_uvw(uvw, half_of(bB, 0), lane), g,
                                             ws.st[0][0], guv, lane, status, false);
-    Issued iB1 = issue_rows<RowStage, !T2D>(half_of(bB, 1), load_uvw(uvw, half_of(bB, 1), lane), g,
+    Issued iB1 = issue_rows<RowStage, !T2D, SMALL>(half_of(bB, 1), load_uvw(uvw, half_of(bB, 1), lane), g,
                                             ws.st[0][1], guv, lane, status, true);
     float2 yB0 = load_y(vis_in, half_of(bB, 0), lane), yB1 = load_y(vis_in, half_of(bB, 1), lane);
     Batch bC = claimer.advance(bB);
@@ -261,9 +273,9 @@ adjoint_kernel(const Geometry g, const double *__restrict__ uvw, const float2 *_
         const int sA = stage;
         bB = bC;
         if (bB.n > 0) {
-            iB0 = issue_rows<RowStage, !T2D>(half_of(bB, 0), cC0, g, ws.st[sA ^ 1][0], guv, lane, status,
+            iB0 = issue_rows<RowStage, !T2D, SMALL>(half_of(bB, 0), cC0, g, ws.st[sA ^ 1][0], guv, lane, status,
                                              false);
-            iB1 = issue_rows<RowStage, !T2D>(half_of(bB, 1), cC1, g, ws.st[sA ^ 1][1], guv, lane, status,
+            iB1 = issue_rows<RowStage, !T2D, SMALL>(half_of(bB, 1), cC1, g, ws.st[sA ^ 1][1], guv, lane, status,
                                              true);
             yB0 = load_y(vis_in, half_of(bB, 0), lane);
             yB1 = load_y(vis_in, half_of(bB, 1), lane);
@@ -292,6 +304,8 @@ adjoint_kernel(const Geometry g, const double *__restrict__ uvw, const float2 *_
     }
     if (rs.key >= 0)
         flush<kVec4>(rs.T, ws, rs.sub_s, rs.key, rs.fw, g, wtab, gwt, p, j);
+    if (checks)
+        check_offsets(pieces, status, lane);
 }
 
 size_t smem_bytes(const degrid_plan *p)
@@ -299,14 +313,19 @@ size_t smem_bytes(const degrid_plan *p)
     return wtable_bytes_host(p->geo) + sizeof(WarpSmem) * (size_t)p->warps_per_block;
 }
 
-// The kernel instance for a 2D table (or not) and vector reductions (or not).
-using AdjointKernel = decltype(&adjoint_kernel<false, false>);
+// The kernel instance for a 2D table (or not), vector reductions (or not) and
+// pieces (or a chunk table).
+using AdjointKernel = decltype(&adjoint_kernel<false, false, false>);
 
-AdjointKernel kernel_for(const degrid_plan *p, bool vec4)
+int instance(const degrid_plan *p, bool vec4, bool small) { return (p->guv2 ? 4 : 0) + (vec4 ? 2 : 0) + (small ? 1 : 0); }
+
+AdjointKernel kernel_for(int k)
 {
-    if (p->guv2)
-        return vec4 ? adjoint_kernel<true, true> : adjoint_kernel<true, false>;
-    return vec4 ? adjoint_kernel<false, true> : adjoint_kernel<false, false>;
+    static constexpr AdjointKernel table[8] = {
+        adjoint_kernel<false, false, false>, adjoint_kernel<false, false, true>, adjoint_kernel<false, true, false>,
+        adjoint_kernel<false, true, true>,   adjoint_kernel<true, false, false>, adjoint_kernel<true, false, true>,
+        adjoint_kernel<true, true, false>,   adjoint_kernel<true, true, true>};
+    return table[k];
 }
 
 // Vector reductions need every element's 32 bytes of w planes 16-byte
@@ -317,44 +336,43 @@ bool vec4_ok(const degrid_plan *p, const void *sub_out)
     return p->geo.nz == kW && (reinterpret_cast<uintptr_t>(sub_out) & 15u) == 0;
 }
 
-// Dynamic shared memory opened so far for the plan's kernel instance on its device.
-std::atomic<size_t> &smem_record(const degrid_plan *p, bool vec4)
+// Dynamic shared memory opened so far for a kernel instance on the plan's device.
+std::atomic<size_t> &smem_record(const degrid_plan *p, int k)
 {
-    static std::atomic<size_t> table[4][kMaxDevices];
-    return dg_smem_record(table[(p->guv2 ? 2 : 0) + (vec4 ? 1 : 0)], p->device);
+    static std::atomic<size_t> table[8][kMaxDevices];
+    return dg_smem_record(table[k], p->device);
 }
 
 }  // namespace
 }  // namespace dg
 
 cudaError_t dg_launch_adjoint(degrid_plan *p, cudaStream_t st, const double *uvw,
-                              const int64_t *vis_offsets, const float *vis_in,
+                              const dg::Pieces &pieces, const float *vis_in,
                               float *sub_out, int grid_blocks)
 {
     using namespace dg;
-    (void)vis_offsets;
     Schedule sched{p->chunks, p->n_chunks, p->work_counter};
     const size_t smem = smem_bytes(p);
-    const bool vec4 = vec4_ok(p, sub_out);
-    const AdjointKernel kernel = kernel_for(p, vec4);
-    const cudaError_t e = dg_open_smem(smem_record(p, vec4), kernel, smem);
+    const int k = instance(p, vec4_ok(p, sub_out), pieces.per_warp > 0);
+    const AdjointKernel kernel = kernel_for(k);
+    const cudaError_t e = dg_open_smem(smem_record(p, k), kernel, smem);
     if (e != cudaSuccess)
         return e;
     return launch_pdl(kernel, dim3(grid_blocks), dim3(p->warps_per_block * kWarp), smem, st, p->geo, uvw,
                       reinterpret_cast<const float2 *>(vis_in), (const float *)p->guv, (const float *)p->gw,
-                      sched, reinterpret_cast<float2 *>(sub_out), p->status, (const float *)p->guv2);
+                      sched, reinterpret_cast<float2 *>(sub_out), p->status, (const float *)p->guv2, pieces);
 }
 
-// Resident CTAs per SM of the instance an aligned output would run (both
-// instances have the same launch bounds and shared memory).
+// Resident CTAs per SM of the instance an aligned output would run (all
+// instances of a table kind have the same launch bounds and shared memory).
 int dg_max_blocks_per_sm_adjoint(degrid_plan *p)
 {
     using namespace dg;
     int n = 0;
     const size_t smem = smem_bytes(p);
-    const bool vec4 = p->geo.nz == kW;
-    const AdjointKernel kernel = kernel_for(p, vec4);
-    if (dg_open_smem(smem_record(p, vec4), kernel, smem) != cudaSuccess)
+    const int k = instance(p, p->geo.nz == kW, false);
+    const AdjointKernel kernel = kernel_for(k);
+    if (dg_open_smem(smem_record(p, k), kernel, smem) != cudaSuccess)
         return 1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, p->warps_per_block * kWarp, smem) !=
         cudaSuccess)

@@ -77,9 +77,10 @@ struct Step {
     float2 *out;
 };
 
-// Steps of the chunks a warp claims.
+// Steps of the chunks (or pieces) a warp claims.
+template <class Claim>
 struct Steps {
-    ClaimerT<kStepVis> claimer;
+    Claim claimer;
     const double *uvw;          // this lane's offset included
     float2 *out;
 
@@ -153,7 +154,7 @@ __device__ __forceinline__ void store_points(MSlot &slot, const float2 (&m)[2], 
 struct Vis2 {
     int key[2];         // footprint start, -1: invalid or past the end of the step
     int fw[2];          // w row
-    int ru[2], rv[2];   // g_u and g_v rows
+    int ru[2], rv[2];   // g_u and g_v rows (-1 with key -1)
 };
 
 __device__ __forceinline__ Vis2 snap_step(const Step &b, const Coords3 (&c)[2], const Geometry &g,
@@ -172,8 +173,8 @@ __device__ __forceinline__ Vis2 snap_step(const Step &b, const Coords3 (&c)[2], 
 #endif
         r.key[h] = valid ? (vc.y0 * g.nx + vc.x0) * g.nz + vc.z0 : -1;
         r.fw[h] = valid ? vc.fw : 0;
-        r.ru[h] = valid ? vc.fu : 0;
-        r.rv[h] = valid ? vc.fv : 0;
+        r.ru[h] = valid ? vc.fu : -1;
+        r.rv[h] = valid ? vc.fv : -1;
         bad[h] = in && !valid;
     }
     if (__any_sync(kFull, bad[0] || bad[1])) {
@@ -190,7 +191,10 @@ struct Row8 {
 };
 
 // Starts the copies of the step's g_u and g_v rows (two lanes per 32-byte
-// row, so each row is one request; one cp.async group).
+// row, so each row is one request; one cp.async group).  Lanes without a
+// valid visibility copy nothing and drop what they sum from the stale stage:
+// one row for all of them made the partial steps of small calls queue up at
+// one sector of L2 (20,000 visibilities in steps of 16: 28 us against 5).
 __device__ __forceinline__ void copy_rows(RowStage (&st)[2], const Vis2 &s, const float *__restrict__ guv, int lane)
 {
     const int half = lane & 1;
@@ -201,6 +205,8 @@ __device__ __forceinline__ void copy_rows(RowStage (&st)[2], const Vis2 &s, cons
             const int row = (lane >> 1) + 16 * m;
             const int xu = __shfl_sync(kFull, s.ru[h], row);
             const int xv = __shfl_sync(kFull, s.rv[h], row);
+            if (xu < 0)
+                continue;
             cp_async16(smem_u32(&st[h].u[row][RowStage::slot(row, half)]), guv + (size_t)xu * kUVRow + 4 * half);
             cp_async16(smem_u32(&st[h].v[row][RowStage::slot(row, half)]), guv + (size_t)xv * kUVRow + 4 * half);
         }
@@ -387,12 +393,13 @@ __device__ __forceinline__ void sum_runs(float2 (&V)[2], MCache &mc, WarpSmem &w
     }
 }
 
-template <int DT, bool COMP>
+// SMALL: by pieces, without a chunk table.
+template <int DT, bool COMP, bool SMALL>
 __global__ void __launch_bounds__(kMaxWarps * kWarp, 2)
 degrid_kernel(const Geometry g, const void *__restrict__ subgrids, const float *__restrict__ scale,
               const double *__restrict__ uvw, const float *__restrict__ guv,
               const float *__restrict__ gwt, const Schedule sched, float2 *__restrict__ vis_out,
-              DeviceStatus *__restrict__ status, const bool vec_ok, const bool prefetch_uvw)
+              DeviceStatus *__restrict__ status, const bool vec_ok, const bool prefetch_uvw, const Pieces pieces)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     // [w table (optional)] [one WarpSmem per warp]
@@ -405,12 +412,21 @@ degrid_kernel(const Geometry g, const void *__restrict__ subgrids, const float *
     // coordinates read in place from host memory are not (the host link
     // bounds those calls, and one batch of lead hides its latency)
     pdl_wait();                         // the chunk table is complete
-    Steps steps{ClaimerT<kStepVis>(sched, lane, Prefetch{prefetch_uvw ? uvw : nullptr, 3 * (int)sizeof(double),
-                                                         nullptr, 0}),
-                uvw + 3 * lane, vis_out + lane};
+    const auto claimer = [&] {
+        if constexpr (SMALL)
+            return PieceClaimerT<kStepVis>(pieces, lane);
+        else
+            return ClaimerT<kStepVis>(sched, lane, Prefetch{prefetch_uvw ? uvw : nullptr, 3 * (int)sizeof(double),
+                                                            nullptr, 0});
+    };
+    Steps<decltype(claimer())> steps{claimer(), uvw + 3 * lane, vis_out + lane};
+    const bool checks = SMALL && blockIdx.x == 0 && threadIdx.x < kWarp;
     Step pA = steps.claim();            // the step being summed
-    if (pA.n == 0)
+    if (pA.n == 0) {
+        if (checks)
+            check_offsets(pieces, status, lane);
         return;
+    }
     Coords3 c[2];
     load_coords(c, pA, lane);
     Vis2 vA = snap_step(pA, c, g, status, lane);
@@ -457,7 +473,8 @@ degrid_kernel(const Geometry g, const void *__restrict__ subgrids, const float *
         pA = pB;
         pB = pC;
     }
-    cp_async_wait<0>();
+    if (checks)
+        check_offsets(pieces, status, lane);
 }
 
 size_t smem_bytes(const degrid_plan *p, int warps)
@@ -466,20 +483,20 @@ size_t smem_bytes(const degrid_plan *p, int warps)
 }
 
 // Dynamic shared memory opened so far for a kernel instance on a device.
-template <int DT, bool COMP>
+template <int DT, bool COMP, bool SMALL>
 std::atomic<size_t> &smem_record(int device)
 {
     static std::atomic<size_t> table[kMaxDevices];
     return dg_smem_record(table, device);
 }
 
-template <int DT, bool COMP>
+template <int DT, bool COMP, bool SMALL>
 cudaError_t launch(degrid_plan *p, cudaStream_t st, const void *subgrids, const float *scale,
-                   const double *uvw, float2 *out, const Schedule &sched, int grid_blocks)
+                   const double *uvw, float2 *out, const Schedule &sched, const Pieces &pieces, int grid_blocks)
 {
     const int threads = p->warps_per_block * kWarp;
     const size_t smem = smem_bytes(p, p->warps_per_block);
-    cudaError_t e = dg_open_smem(smem_record<DT, COMP>(p->device), degrid_kernel<DT, COMP>,
+    cudaError_t e = dg_open_smem(smem_record<DT, COMP, SMALL>(p->device), degrid_kernel<DT, COMP, SMALL>,
                                  smem);
     if (e != cudaSuccess)
         return e;
@@ -487,20 +504,20 @@ cudaError_t launch(degrid_plan *p, cudaStream_t st, const void *subgrids, const 
     // elements per 16 bytes
     const bool vec_ok = (reinterpret_cast<uintptr_t>(subgrids) & 15) == 0 &&
                         p->geo.nz % Storage<DT>::kQuad == 0;
-    return launch_pdl(degrid_kernel<DT, COMP>, dim3(grid_blocks), dim3(threads), smem, st,
+    return launch_pdl(degrid_kernel<DT, COMP, SMALL>, dim3(grid_blocks), dim3(threads), smem, st,
                       p->geo, subgrids, scale, uvw, (const float *)p->guv, (const float *)p->gw, sched, out,
-                      p->status, vec_ok, !p->host_inputs);
+                      p->status, vec_ok, !p->host_inputs, pieces);
 }
 
-template <int DT, bool COMP>
+template <int DT, bool COMP, bool SMALL>
 int max_blocks(degrid_plan *p)
 {
     int n = 0;
     const size_t smem = smem_bytes(p, p->warps_per_block);
-    if (dg_open_smem(smem_record<DT, COMP>(p->device), degrid_kernel<DT, COMP>, smem) !=
+    if (dg_open_smem(smem_record<DT, COMP, SMALL>(p->device), degrid_kernel<DT, COMP, SMALL>, smem) !=
         cudaSuccess)
         return 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, degrid_kernel<DT, COMP>,
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, degrid_kernel<DT, COMP, SMALL>,
                                                       p->warps_per_block * kWarp, smem) != cudaSuccess)
         return 1;
     return n > 0 ? n : 1;
@@ -511,27 +528,28 @@ int max_blocks(degrid_plan *p)
 // kernels of their own.
 template <int DT>
 cudaError_t launch_dt(degrid_plan *p, cudaStream_t st, const void *subgrids, const float *scale,
-                      const double *uvw, float2 *out, const Schedule &sched, int grid_blocks)
+                      const double *uvw, float2 *out, const Schedule &sched, const Pieces &pieces, int grid_blocks)
 {
-    return p->compensated ? launch<DT, true>(p, st, subgrids, scale, uvw, out, sched, grid_blocks)
-                          : launch<DT, false>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
+    const auto run = [&](auto fn) { return fn(p, st, subgrids, scale, uvw, out, sched, pieces, grid_blocks); };
+    if (pieces.per_warp > 0)
+        return p->compensated ? run(launch<DT, true, true>) : run(launch<DT, false, true>);
+    return p->compensated ? run(launch<DT, true, false>) : run(launch<DT, false, false>);
 }
 
 template <int DT>
 int max_blocks_dt(degrid_plan *p)
 {
-    return p->compensated ? max_blocks<DT, true>(p) : max_blocks<DT, false>(p);
+    return p->compensated ? max_blocks<DT, true, false>(p) : max_blocks<DT, false, false>(p);
 }
 
 }  // namespace
 }  // namespace dg
 
 cudaError_t dg_launch_degrid(degrid_plan *p, cudaStream_t st, const void *subgrids,
-                             const float *scale, const double *uvw, const int64_t *vis_offsets,
+                             const float *scale, const double *uvw, const dg::Pieces &pieces,
                              float *out_f, int grid_blocks)
 {
     using namespace dg;
-    (void)vis_offsets;
     if (p->guv2)
         return dg_launch_degrid_2d(p, st, subgrids, scale, uvw, out_f, grid_blocks);
     if (p->direct_runs < DG_DIRECT_RUNS_NEVER)
@@ -540,11 +558,11 @@ cudaError_t dg_launch_degrid(degrid_plan *p, cudaStream_t st, const void *subgri
     float2 *out = reinterpret_cast<float2 *>(out_f);
     switch (p->dtype) {
     case DG_C64:
-        return launch_dt<DG_C64>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
+        return launch_dt<DG_C64>(p, st, subgrids, scale, uvw, out, sched, pieces, grid_blocks);
     case DG_C32_F16:
-        return launch_dt<DG_C32_F16>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
+        return launch_dt<DG_C32_F16>(p, st, subgrids, scale, uvw, out, sched, pieces, grid_blocks);
     case DG_C32_BF16:
-        return launch_dt<DG_C32_BF16>(p, st, subgrids, scale, uvw, out, sched, grid_blocks);
+        return launch_dt<DG_C32_BF16>(p, st, subgrids, scale, uvw, out, sched, pieces, grid_blocks);
     }
     return cudaErrorInvalidValue;
 }

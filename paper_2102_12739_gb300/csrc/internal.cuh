@@ -189,6 +189,15 @@ struct Schedule {
     int *work_counter;              // zeroed by the scheduler before every launch
 };
 
+// Work of a small call, without a chunk table: warp k of the grid takes
+// visibilities [k per_warp, (k + 1) per_warp) of whatever lists they are in.
+struct Pieces {
+    const int64_t *offs;
+    int n_subgrids;
+    int per_warp;                   // 0: the call has a chunk table
+    int64_t n_vis;
+};
+
 // Bound on the polls of any device-side wait (mbarrier phase); a wait that
 // exceeds it records kFlagTimeout and the warp stops working.
 constexpr int kSpinLimit = 1 << 22;
@@ -343,11 +352,17 @@ inline int dg_small_items(int chunk) { return chunk > 64 ? 64 : 0; }
 
 // Kernel launchers (one per translation unit).
 cudaError_t dg_launch_degrid(degrid_plan *p, cudaStream_t st, const void *subgrids,
-                             const float *scale, const double *uvw,
-                             const int64_t *vis_offsets, float *vis_out, int grid_blocks);
+                             const float *scale, const double *uvw, const dg::Pieces &pieces,
+                             float *vis_out, int grid_blocks);
 cudaError_t dg_launch_adjoint(degrid_plan *p, cudaStream_t st, const double *uvw,
-                              const int64_t *vis_offsets, const float *vis_in,
+                              const dg::Pieces &pieces, const float *vis_in,
                               float *sub_out, int grid_blocks);
+// Whether the degridding kernel of the plan can work by pieces (those with a
+// 2D table or the direct arm cannot).
+inline bool dg_degrid_takes_pieces(const degrid_plan *p)
+{
+    return !p->guv2 && p->direct_runs >= DG_DIRECT_RUNS_NEVER;
+}
 cudaError_t dg_launch_coords(degrid_plan *p, cudaStream_t st, const double *uvw,
                              int64_t n_vis, int32_t *coords_out);
 cudaError_t dg_launch_gather(degrid_plan *p, cudaStream_t st, const void *subgrids, int n_subgrids,

@@ -16,10 +16,6 @@
 
 #include "internal.cuh"
 
-cudaError_t dg_launch_degrid(degrid_plan *p, cudaStream_t st, const void *subgrids,
-                             const float *scale, const double *uvw,
-                             const int64_t *vis_offsets, float *vis_out, int grid_blocks);
-
 namespace {
 
 // Scratch layout, in bytes from the start of the array.
@@ -163,6 +159,6 @@ extern "C" dg_status degrid_execute_noalloc(void *stream, int nx, int ny, int nz
         blocks = useful;
     if (blocks < 1)
         blocks = 1;
-    return from_cuda(dg_launch_degrid(&p, s, subgrids, subgrid_scale, uvw, vis_offsets, vis_out,
+    return from_cuda(dg_launch_degrid(&p, s, subgrids, subgrid_scale, uvw, dg::Pieces{}, vis_out,
                                       (int)blocks));
 }

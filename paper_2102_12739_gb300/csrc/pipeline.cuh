@@ -145,6 +145,77 @@ struct ClaimerT {
 
 using Claimer = ClaimerT<kBatch>;
 
+// The warp's piece of a small call (Pieces), as the batches of the lists it
+// overlaps: the same interface as ClaimerT.  Every list is looked at, so
+// malformed offsets give the batches a chunk table would hold.
+template <int kStep>
+struct PieceClaimerT {
+    const Pieces &pieces;
+    int lane;
+    long long first, last;      // the piece
+    long long lo, hi;           // lane: its list's part of the piece (group of 32 lists before `next`)
+    int next;                   // lists not yet looked at
+    unsigned todo;              // lists of the group with visibilities left to batch
+
+    __device__ PieceClaimerT(const Pieces &p, int lane_) : pieces(p), lane(lane_), lo(0), hi(0), next(0), todo(0)
+    {
+        const long long k = (long long)blockIdx.x * (blockDim.x / kWarp) + threadIdx.x / kWarp;
+        first = k * p.per_warp;
+        last = min(first + p.per_warp, (long long)p.n_vis);
+    }
+
+    __device__ Batch claim()
+    {
+        while (todo == 0) {
+            if (next >= pieces.n_subgrids || first >= last)
+                return Batch{0, 0, 0, 0};
+            const int s = next + lane;
+            lo = hi = 0;
+            if (s < pieces.n_subgrids) {
+                const long long a = pieces.offs[s], b = pieces.offs[s + 1];
+                if (a >= 0 && a <= b && b <= pieces.n_vis) {
+                    lo = max(a, first);
+                    hi = min(b, last);
+                }
+            }
+            todo = __ballot_sync(kFull, lo < hi);
+            next += kWarp;
+        }
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1;
+        Batch b;
+        b.s = next - kWarp + src;
+        b.b0 = __shfl_sync(kFull, lo, src);
+        b.end = __shfl_sync(kFull, hi, src);
+        b.n = (int)min((long long)kStep, b.end - b.b0);
+        return b;
+    }
+
+    __device__ Batch advance(const Batch &b)
+    {
+        if (b.n == 0)
+            return b;
+        Batch nb = b;
+        nb.b0 = b.b0 + kStep;
+        if (nb.b0 >= b.end)
+            return claim();
+        nb.n = (int)min((long long)kStep, b.end - nb.b0);
+        return nb;
+    }
+};
+
+// Records malformed offsets, as the scheduling kernel does (one warp).
+__device__ __forceinline__ void check_offsets(const Pieces &p, DeviceStatus *status, int lane)
+{
+    bool bad = lane == 0 && (p.offs[0] != 0 || p.offs[p.n_subgrids] != p.n_vis);
+    for (int s = lane; s < p.n_subgrids; s += kWarp) {
+        const long long a = p.offs[s], b = p.offs[s + 1];
+        bad = bad || !(a >= 0 && a <= b && b <= p.n_vis);
+    }
+    if (__any_sync(kFull, bad) && lane == 0)
+        atomicOr(&status->flags, kFlagOffsets);
+}
+
 // The visibilities [b0 + 32h, b0 + 32h + 32) of a batch of 64.
 __device__ __forceinline__ Batch half_of(const Batch &b, int h)
 {
@@ -201,8 +272,11 @@ struct Issued {
 // Stage 2 of a degridding batch: snap, and copy the g_u / g_v rows into the
 // stage (2 lanes per 32-byte row, so each row is one request).
 // With kRows = false (a 2D G_uv table, read by the summing lanes themselves)
-// no rows are staged; the weight block index is kept instead.
-template <class Stage, bool kRows = true>
+// no rows are staged; the weight block index is kept instead.  kSpread: lanes
+// without a valid visibility copy the rows of one that has one, for callers
+// whose batches are often partial (with row 0 for all of them these copies
+// queue up at one sector of L2).
+template <class Stage, bool kRows = true, bool kSpread = false>
 __device__ __forceinline__ Issued issue_rows(const Batch &b, const Coords3 &c, const Geometry &g,
                                              Stage &S, const float *__restrict__ guv, int lane,
                                              DeviceStatus *status, bool commit = true)
@@ -217,7 +291,16 @@ __device__ __forceinline__ Issued issue_rows(const Batch &b, const Coords3 &c, c
     Issued r;
     r.key = valid ? (vc.y0 * g.nx + vc.x0) * g.nz + vc.z0 : -1;
     r.fw = valid ? vc.fw : 0;
-    const int fu = valid ? vc.fu : 0, fv = valid ? vc.fv : 0;
+    int fu = valid ? vc.fu : 0, fv = valid ? vc.fv : 0;
+    if (kSpread) {
+        const unsigned have = __ballot_sync(kFull, valid);
+        if (have != kFull && have != 0) {
+            const int src = __ffs(have) - 1;
+            const int su = __shfl_sync(kFull, fu, src), sv = __shfl_sync(kFull, fv, src);
+            fu = valid ? fu : su;
+            fv = valid ? fv : sv;
+        }
+    }
     r.key0 = __shfl_sync(kFull, r.key, 0);
     r.fw0 = __shfl_sync(kFull, r.fw, 0);
     // lanes past the end of the batch compute values nobody stores

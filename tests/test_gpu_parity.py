@@ -1182,3 +1182,67 @@ def test_steps_of_many_runs(dtype, comp, nz):
     assert np.all(outs[0][bad] == 0)
     for o in outs[1:]:
         np.testing.assert_array_equal(o.view(np.uint64), outs[0].view(np.uint64))
+
+
+@pytest.mark.parametrize("counts", [
+    [1], [16], [17, 0, 0, 47], [63], [64], [65], [3] * 100, [0, 5] * 40 + [1000], [20000], [4000, 0, 3, 9000, 1],
+    [7] * 256, [7] * 257,                                       # the most lists of a call by pieces, and one more
+])
+def test_small_calls_by_pieces(counts):
+    # pieces that span several lists, empty lists, lists cut by pieces, more
+    # than 32 lists, invalid visibilities: degridding bit for bit and gridding
+    # against a plan whose two CTA warps cannot hold the call (a chunk table)
+    d = dev()
+    shape = (40, 48, 4)
+    w = small_workload(counts, kind="mixed", shape=shape, seed=95)
+    uvw_np = w.uvw.copy()
+    uvw_np[:: max(1, len(uvw_np) // 7)] += np.array([0.0, 0.0, 50.0])
+    n_bad = len(uvw_np[:: max(1, len(uvw_np) // 7)])
+    sub_np = synth.subgrid_stack(len(counts), shape=shape)
+    sub = torch.from_numpy(sub_np).to(d)
+    uvw, offs = torch.from_numpy(uvw_np).to(d), torch.from_numpy(w.vis_offsets).to(d)
+    y = synth.adjoint_vis(w.n_vis)
+    ref, bad = oracle.degrid(G_UV, G_W, sub_np.astype(np.complex128), uvw_np, w.vis_offsets)
+    gref, _ = oracle.grid(G_UV, G_W, shape, len(counts), uvw_np, w.vis_offsets, y)
+    assert bad == n_bad
+    with dg.DegridPlan(shape=shape, device=d) as p:
+        got = p.degrid(sub, uvw, offs).cpu().numpy()
+        assert p.status() == n_bad
+        grid = p.grid(torch.from_numpy(y).to(d), uvw, offs, len(counts)).cpu().numpy()
+        assert p.status() == n_bad
+        # a larger call of the same lists, twice over, goes by the chunk table
+        reps = 1 + 200000 // w.n_vis
+        big = torch.from_numpy(np.tile(uvw_np, (reps, 1))).to(d)
+        many = torch.from_numpy(np.concatenate([[0], np.full(len(counts) - 1, 0), [w.n_vis * reps]])).to(d)
+        if len(counts) == 1:
+            tab = p.degrid(sub, big, many).cpu().numpy()[: w.n_vis]
+            np.testing.assert_array_equal(got.view(np.uint64), tab.view(np.uint64))
+    scale = max(float(np.linalg.norm(ref)), 1e-30)
+    assert np.linalg.norm(got - ref) <= 2e-6 * scale
+    assert np.linalg.norm(grid - gref) <= 2e-6 * max(float(np.linalg.norm(gref)), 1e-30)
+
+
+def test_small_calls_report_malformed_offsets():
+    # decreasing, negative and too large offsets of a call by pieces: flagged,
+    # the valid lists still done, nothing written outside them
+    d = dev()
+    w = small_workload([100, 100, 100], shape=SHAPE, seed=96)
+    sub, uvw, _ = upload(w, synth.subgrid_stack(3))
+    with dg.DegridPlan(device=d) as p:
+        full = p.degrid(sub, uvw, torch.tensor([0, 100, 200, 300], device=d)).cpu().numpy()
+        assert p.status() == 0
+        for offs in ([0, 150, 100, 300], [0, -5, 200, 300], [0, 100, 400, 300], [0, 100, 200, 250], [10, 100, 200, 300]):
+            out = torch.full((300,), 7.0 + 3.0j, dtype=torch.complex64, device=d)
+            p.degrid(sub, uvw, torch.tensor(offs, dtype=torch.int64, device=d), out=out)
+            with pytest.raises(dg.DegridError) as e:
+                p.status()
+            assert e.value.status == dg.DG_ERR_OFFSETS
+            got = out.cpu().numpy()
+            for s in range(3):
+                if offs[s] == 100 * s and offs[s + 1] == 100 * (s + 1):
+                    np.testing.assert_array_equal(got[100 * s: 100 * (s + 1)], full[100 * s: 100 * (s + 1)])
+            covered = np.zeros(300, dtype=bool)
+            for a, b in zip(offs[:-1], offs[1:]):
+                if 0 <= a <= b <= 300:
+                    covered[a:b] = True
+            assert np.all(got[~covered] == 7.0 + 3.0j)
