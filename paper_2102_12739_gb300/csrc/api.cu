@@ -208,33 +208,42 @@ bool tiled(degrid_plan *p, cudaStream_t st, dg::TileShape shape, int n_subgrids,
 }
 
 // The pieces of a call too small to need a chunk table: one step of at most
-// kPieceMost visibilities for every resident warp, which saves the scheduling
+// `most` visibilities for every resident warp, which saves the scheduling
 // kernel's launch and run (20,000 visibilities on a line: 12.3 -> 4.6 us of
 // GPU time).  If there are not enough visibilities for all warps, a piece has
 // `least` of them.  Few enough lists for every warp to look at all of them.
 // per_warp 0: not such a call.
-constexpr int kPieceMost = 64;
+constexpr int kPieceMost = 64;          // one step
 constexpr int kPieceLists = 256;
+
+// The library variant that tests the gather kernel's bounded wait keeps small
+// calls of plans with the gather setting on that kernel.
+#ifdef DG_GATHER_SUM_WAIT_POLLS
+constexpr bool kKeepGather = true;
+#else
+constexpr bool kKeepGather = false;
+#endif
 
 // Degridding: short pieces let many warps build the footprints of a list of
 // short runs (100 lists of 200: 14 us in pieces of 16, 28 of 64).
 constexpr int kDegridPieceLeast = 16;
 
-// Gridding: a piece ends with adds into the subgrid, so pieces are as long as
-// the lists (a list of 20,000: 10 us in pieces of 64, 25 of 16; 100 lists of
-// 10: 127 us in pieces of 16, 157 of 64).
-int grid_piece_least(int n_subgrids, int64_t n_vis)
-{
-    const int64_t list = (n_vis + n_subgrids - 1) / n_subgrids;
-    return list < kPieceMost ? (int)((list + 7) / 8 * 8) : kPieceMost;
-}
+// Gridding the same, although a piece ends with adds into the subgrid (8
+// lists of 125: 21 us in pieces of 8, 50 of 64; a list of 20,000: 11 and 10).
+constexpr int kGridPieceLeast = 8;
+
+// The most visibilities per warp.  Scattered ones (the gather setting) are
+// gridded faster by the scatter kernel from about 80,000 on; up to the limit
+// they are degridded faster this way than by the gather kernel (20,000 on one
+// subgrid: 15 us against 40).
+int grid_piece_most(const degrid_plan *p) { return p->gather ? kPieceMost / 2 : kPieceMost; }
 
 dg::Pieces pieces_of(const degrid_plan *p, const int64_t *vis_offsets, int n_subgrids, int64_t n_vis, int max_per_sm,
-                     int least)
+                     int least, int most)
 {
     const int per_sm = p->blocks_per_sm > 0 && p->blocks_per_sm < max_per_sm ? p->blocks_per_sm : max_per_sm;
     const int64_t warps = (int64_t)p->sm_count * per_sm * p->warps_per_block;
-    const bool small = n_subgrids <= kPieceLists && n_vis <= warps * kPieceMost;
+    const bool small = n_subgrids <= kPieceLists && n_vis <= warps * most;
     const int64_t share = (n_vis + warps - 1) / warps;
     return dg::Pieces{vis_offsets, n_subgrids, small ? (int)(share > least ? share : least) : 0, n_vis};
 }
@@ -628,14 +637,13 @@ dg_status degrid_execute(degrid_plan_t p, void *stream, int n_subgrids, const vo
         timer.stop();
         return from_cuda(e);
     }
-    const bool gather = p->gather && tma_rows_fit(p, n_subgrids);
+    if (p->max_blocks_degrid == 0)
+        p->max_blocks_degrid = dg_max_blocks_per_sm_degrid(p);
     dg::Pieces pieces{};
-    if (!gather) {
-        if (p->max_blocks_degrid == 0)
-            p->max_blocks_degrid = dg_max_blocks_per_sm_degrid(p);
-        if (dg_degrid_takes_pieces(p))
-            pieces = pieces_of(p, vis_offsets, n_subgrids, n_vis, p->max_blocks_degrid, kDegridPieceLeast);
-    }
+    if (dg_degrid_takes_pieces(p) && !(kKeepGather && p->gather))
+        pieces = pieces_of(p, vis_offsets, n_subgrids, n_vis, p->max_blocks_degrid, kDegridPieceLeast,
+                           kPieceMost);
+    const bool gather = p->gather && pieces.per_warp == 0 && tma_rows_fit(p, n_subgrids);
     cudaError_t e = cudaSuccess;
     if (pieces.per_warp == 0)
         e = dg::launch_schedule(s, vis_offsets, n_subgrids, n_vis, chunk, dg_small_items(chunk), p->prefix,
@@ -687,7 +695,11 @@ dg_status grid_adjoint_execute(degrid_plan_t p, void *stream, int n_subgrids, co
     dg_status st = ensure_capacity(p, n_subgrids, n_vis, chunk);
     if (st != DG_OK)
         return st;
-    if (aligned(sub_out, 16) && tiled(p, s, kGridTile, n_subgrids, n_vis)) {
+    if (p->max_blocks_adjoint == 0)
+        p->max_blocks_adjoint = dg_max_blocks_per_sm_adjoint(p);
+    const dg::Pieces pieces = pieces_of(p, vis_offsets, n_subgrids, n_vis, p->max_blocks_adjoint,
+                                        kGridPieceLeast, grid_piece_most(p));
+    if (pieces.per_warp == 0 && aligned(sub_out, 16) && tiled(p, s, kGridTile, n_subgrids, n_vis)) {
         KernelTimer timer(p, s);
         dg::Bins bins;
         cudaError_t e = dg_bins_sort(p, s, kGridTile, n_subgrids, n_vis, uvw, vis_offsets, nullptr, &bins);
@@ -696,14 +708,7 @@ dg_status grid_adjoint_execute(degrid_plan_t p, void *stream, int n_subgrids, co
         timer.stop();
         return from_cuda(e);
     }
-    const bool scatter = p->gather && aligned(sub_out, 16) && tma_rows_fit(p, n_subgrids);
-    dg::Pieces pieces{};
-    if (!scatter) {
-        if (p->max_blocks_adjoint == 0)
-            p->max_blocks_adjoint = dg_max_blocks_per_sm_adjoint(p);
-        pieces = pieces_of(p, vis_offsets, n_subgrids, n_vis, p->max_blocks_adjoint,
-                           grid_piece_least(n_subgrids, n_vis));
-    }
+    const bool scatter = p->gather && pieces.per_warp == 0 && aligned(sub_out, 16) && tma_rows_fit(p, n_subgrids);
     cudaError_t e = cudaSuccess;
     if (pieces.per_warp == 0)
         e = dg::launch_schedule(s, vis_offsets, n_subgrids, n_vis, chunk, dg_small_items(chunk), p->prefix,

@@ -273,9 +273,9 @@ struct Issued {
 // stage (2 lanes per 32-byte row, so each row is one request).
 // With kRows = false (a 2D G_uv table, read by the summing lanes themselves)
 // no rows are staged; the weight block index is kept instead.  kSpread: lanes
-// without a valid visibility copy the rows of one that has one, for callers
-// whose batches are often partial (with row 0 for all of them these copies
-// queue up at one sector of L2).
+// without a valid visibility copy the rows of one that has one, and a batch
+// without any copies none, for callers whose batches are often partial (with
+// row 0 for all of them these copies queue up at one sector of L2).
 template <class Stage, bool kRows = true, bool kSpread = false>
 __device__ __forceinline__ Issued issue_rows(const Batch &b, const Coords3 &c, const Geometry &g,
                                              Stage &S, const float *__restrict__ guv, int lane,
@@ -292,9 +292,11 @@ __device__ __forceinline__ Issued issue_rows(const Batch &b, const Coords3 &c, c
     r.key = valid ? (vc.y0 * g.nx + vc.x0) * g.nz + vc.z0 : -1;
     r.fw = valid ? vc.fw : 0;
     int fu = valid ? vc.fu : 0, fv = valid ? vc.fv : 0;
+    bool empty = false;
     if (kSpread) {
         const unsigned have = __ballot_sync(kFull, valid);
-        if (have != kFull && have != 0) {
+        empty = have == 0;
+        if (have != kFull && !empty) {
             const int src = __ffs(have) - 1;
             const int su = __shfl_sync(kFull, fu, src), sv = __shfl_sync(kFull, fv, src);
             fu = valid ? fu : su;
@@ -314,7 +316,7 @@ __device__ __forceinline__ Issued issue_rows(const Batch &b, const Coords3 &c, c
     if (lane == 0 && bad)
         atomicAdd(&status->n_invalid, (unsigned long long)__popc(bad));
     r.blk = (fv << g.log2_uv_os) + fu;
-    if (!kRows) {
+    if (!kRows || empty) {
         if (commit)
             cp_async_commit();
         return r;

@@ -247,3 +247,34 @@ def test_a_captured_call_larger_than_the_tiles_workspace():
         second = p.degrid(sub, uvw, offs).cpu().numpy()         # by tiles
         assert p.status() == 0
     np.testing.assert_array_equal(first.view(np.uint64), second.view(np.uint64))
+
+
+@pytest.mark.parametrize("dtype,comp", [("c64", False), ("c64", True), ("f16", False), ("bf16", True)])
+def test_gather_and_scatter_kernels_on_many_lists(dtype, comp):
+    # more lists than a call by pieces takes and too few visibilities for
+    # tiles: every footprint by itself (ragged lists, empty ones, invalid
+    # visibilities), bit for bit the cached path; gridding against the oracle
+    d = dev()
+    shape = (32, 40, 4)
+    rng = np.random.default_rng(5)
+    counts = [int(c) for c in rng.integers(0, 12, 300)] + [700, 0, 513]
+    w = small_workload(counts, kind="scatter", shape=shape, seed=97)
+    uvw_np = w.uvw.copy()
+    uvw_np[::97] = [9.0, 9.0, -4.0]
+    sub_np = synth.subgrid_stack(len(counts), shape=shape)
+    sub = torch.from_numpy(sub_np).to(d)
+    codes, scale = (sub, None) if dtype == "c64" else dg.pack_subgrids(sub, dtype)
+    uvw, offs = torch.from_numpy(uvw_np).to(d), torch.from_numpy(w.vis_offsets).to(d)
+    outs = []
+    for gather in (False, True):
+        with dg.DegridPlan(shape=shape, dtype=dtype, device=d, compensated=comp, gather=gather) as p:
+            outs.append(p.degrid(codes, uvw, offs, scale=scale).cpu().numpy())
+            assert p.status() == len(uvw_np[::97])
+    np.testing.assert_array_equal(bits(outs[0]), bits(outs[1]))
+    if dtype == "c64":
+        y = synth.adjoint_vis(w.n_vis)
+        ref, _ = oracle.grid(G_UV, G_W, shape, len(counts), uvw_np, w.vis_offsets, y)
+        with dg.DegridPlan(shape=shape, device=d, gather=True) as p:
+            out = p.grid(torch.from_numpy(y).to(d), uvw, offs, len(counts)).cpu().numpy()
+            assert p.status() == len(uvw_np[::97])
+        assert rel_l2(out, ref) <= 2e-6
