@@ -228,9 +228,14 @@ constexpr bool kKeepGather = false;
 // short runs (100 lists of 200: 14 us in pieces of 16, 28 of 64).
 constexpr int kDegridPieceLeast = 16;
 
-// Gridding the same, although a piece ends with adds into the subgrid (8
-// lists of 125: 21 us in pieces of 8, 50 of 64; a list of 20,000: 11 and 10).
-constexpr int kGridPieceLeast = 8;
+// Gridding: a run's sum is added into the subgrid in FP32 at the end of its
+// piece, and shorter pieces add more partial sums (pieces of 8 against 64 for
+// 20,000 visibilities of lines and arcs on one subgrid: an error of 2.2e-7
+// against 1.5e-7 to FP64).  So a piece is what a chunk of such a call is.
+// With the gather setting the scatter kernel would add every visibility by
+// itself, so short pieces lose nothing (8 lists of 125: 21 us in pieces of 8,
+// 50 of 64).
+int grid_piece_least(const degrid_plan *p) { return p->gather ? 8 : kPieceMost; }
 
 // The most visibilities per warp.  Scattered ones (the gather setting) are
 // gridded faster by the scatter kernel from about 80,000 on; up to the limit
@@ -698,7 +703,7 @@ dg_status grid_adjoint_execute(degrid_plan_t p, void *stream, int n_subgrids, co
     if (p->max_blocks_adjoint == 0)
         p->max_blocks_adjoint = dg_max_blocks_per_sm_adjoint(p);
     const dg::Pieces pieces = pieces_of(p, vis_offsets, n_subgrids, n_vis, p->max_blocks_adjoint,
-                                        kGridPieceLeast, grid_piece_most(p));
+                                        grid_piece_least(p), grid_piece_most(p));
     if (pieces.per_warp == 0 && aligned(sub_out, 16) && tiled(p, s, kGridTile, n_subgrids, n_vis)) {
         KernelTimer timer(p, s);
         dg::Bins bins;
