@@ -14,9 +14,9 @@
 // at nz consecutive w-planes, stored [y][x][c] like the stack the degridding
 // kernels read.
 //
-// Sizes and plane counts that predict_fft.cu covers take its two kernels
-// (screen and row transforms, column transforms and window).  The others
-// take, per pass of up to P subgrids, three steps on the caller's stream:
+// Sizes that predict_fft.cu covers take its two kernels (screen and row
+// transforms, column transforms and window).  The others take, per pass of up
+// to P subgrids, three steps on the caller's stream:
 //  1. screen_kernel (hand-written): for every pixel and subgrid, the tapered
 //     image times the w-phase screen of each plane and (-1)^(a + b) into a
 //     work buffer [P][nz][N][N].  The phase w (n - 1) runs to hundreds of
@@ -50,7 +50,7 @@ struct subgrid_predict_plan {
     int n, nz, per_pass;
     cufftHandle fft;
     bool fft_ok;
-    dg_predict_fft *fused;      // the fused transform, where there is one for n and nz (the rest is unused then)
+    dg_predict_fft *fused;      // the fused transform, where there is one for n (the rest is unused then)
     float2 *work;       // [per_pass][nz][n][n]
     float2 *nm1;        // [n][n]: n - 1 per pixel as (hi, lo) floats, hi NaN outside the unit circle
 };
@@ -236,7 +236,7 @@ dg_status subgrid_predict_plan_create(subgrid_predict_plan_t *out, int n, int nz
     p->work = nullptr;
     p->nm1 = nullptr;
     p->fused = nullptr;
-    if (dg_predict_fft_supported(n, nz)) {
+    if (dg_predict_fft_supported(n)) {
         const cudaError_t err = dg_predict_fft_create(&p->fused, n, nz, subgrids_per_pass, device);
         if (err != cudaSuccess) {
             delete p;

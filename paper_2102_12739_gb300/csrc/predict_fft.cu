@@ -38,8 +38,7 @@ __global__ void nm1_quadrant_kernel(float2 *__restrict__ nm1, int half, double d
 }  // namespace dg
 
 struct dg_predict_fft {
-    int n, groups;                  // side; plane groups (items) per subgrid
-    int nz;
+    int n, nz;                      // side; planes per subgrid
     int pass;                       // subgrids per pass at most
     int blocks_rows, blocks_cols;   // resident blocks on the device
     float2 *work, *nm1, *tw;
@@ -93,20 +92,20 @@ std::vector<float2> twiddle_table()
     return h;
 }
 
-template <class F>
+template <class F, bool PACKED>
 cudaError_t prepare(dg_predict_fft *p, int device, int sm_count)
 {
     static_assert(F::T % kTileCols == 0, "a thread's columns share their place in the tiles");
     static std::atomic<size_t> rows_smem[kMaxDevices], cols_smem[kMaxDevices];
-    cudaError_t e = dg_open_smem(dg_smem_record(rows_smem, device), rows_kernel<F>, RowsShape<F>::kSmem);
+    cudaError_t e = dg_open_smem(dg_smem_record(rows_smem, device), rows_kernel<F, PACKED>, RowsShape<F>::kSmem);
     if (e == cudaSuccess)
-        e = dg_open_smem(dg_smem_record(cols_smem, device), columns_kernel<F>, ColumnsShape<F>::kSmem);
+        e = dg_open_smem(dg_smem_record(cols_smem, device), columns_kernel<F, PACKED>, ColumnsShape<F>::kSmem);
     int nr = 0, nc = 0;
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nr, rows_kernel<F>, RowsShape<F>::kThreads,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nr, rows_kernel<F, PACKED>, RowsShape<F>::kThreads,
                                                           RowsShape<F>::kSmem);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nc, columns_kernel<F>, ColumnsShape<F>::kThreads,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nc, columns_kernel<F, PACKED>, ColumnsShape<F>::kThreads,
                                                           ColumnsShape<F>::kSmem);
     if (e != cudaSuccess)
         return e;
@@ -119,25 +118,25 @@ cudaError_t prepare(dg_predict_fft *p, int device, int sm_count)
     return e;
 }
 
-template <class F>
+template <class F, bool PACKED>
 cudaError_t rows(const dg_predict_fft *p, cudaStream_t st, int blocks, const RowsArgs &a)
 {
-    return launch_pdl(rows_kernel<F>, dim3(blocks), dim3(RowsShape<F>::kThreads), RowsShape<F>::kSmem, st, a.image,
+    return launch_pdl(rows_kernel<F, PACKED>, dim3(blocks), dim3(RowsShape<F>::kThreads), RowsShape<F>::kSmem, st, a.image,
                       a.taper, (const float2 *)p->nm1, a.w_planes, a.items, (const float2 *)p->tw, p->work,
                       a.first_pass);
 }
 
-template <class F>
+template <class F, bool PACKED>
 cudaError_t columns(const dg_predict_fft *p, cudaStream_t st, int blocks, const ColumnsArgs &a)
 {
-    return launch_pdl(columns_kernel<F>, dim3(blocks), dim3(ColumnsShape<F>::kThreads), ColumnsShape<F>::kSmem, st,
-                      (const float2 *)p->work, a.uv_offsets, a.items, p->nz, (const float2 *)p->tw, a.out);
+    return launch_pdl(columns_kernel<F, PACKED>, dim3(blocks), dim3(ColumnsShape<F>::kThreads), ColumnsShape<F>::kSmem, st,
+                      (const float2 *)p->work, a.uv_offsets, a.items, (const float2 *)p->tw, a.out);
 }
 
-template <class F>
+template <class F, bool PACKED>
 constexpr Variant variant()
 {
-    return Variant{F::N, prepare<F>, rows<F>, columns<F>};
+    return Variant{F::N, prepare<F, PACKED>, rows<F, PACKED>, columns<F, PACKED>};
 }
 
 // <side, points per thread, radices>: few exchanges (two radices, so one,
@@ -145,19 +144,32 @@ constexpr Variant variant()
 // as (32, 16) 355 us, as (16, 16, 2) 441, as (8, 8, 8) 472 for 64 subgrids of
 // four planes; 384 as (24, 4, 4) 91 us, (8, 8, 6) 99, (24, 16) with 48 points
 // per thread 116 for 21 subgrids.
+// PACKED: for one or two planes per subgrid.
+template <bool PACKED>
 constexpr Variant kVariants[] = {
-    variant<LineFft<64, 8, 8, 8>>(),       variant<LineFft<96, 24, 24, 4>>(),   variant<LineFft<128, 16, 16, 8>>(),
-    variant<LineFft<192, 24, 24, 8>>(),    variant<LineFft<256, 16, 16, 16>>(), variant<LineFft<320, 40, 40, 8>>(),
-    variant<LineFft<384, 24, 24, 4, 4>>(), variant<LineFft<400, 20, 20, 20>>(), variant<LineFft<512, 32, 32, 16>>(),
-    variant<LineFft<768, 24, 24, 8, 4>>(), variant<LineFft<1024, 32, 32, 32>>(),
+    variant<LineFft<64, 8, 8, 8>, PACKED>(), variant<LineFft<96, 24, 24, 4>, PACKED>(),
+    variant<LineFft<128, 16, 16, 8>, PACKED>(), variant<LineFft<192, 24, 24, 8>, PACKED>(),
+    variant<LineFft<200, 10, 10, 10, 2>, PACKED>(), variant<LineFft<256, 16, 16, 16>, PACKED>(),
+    variant<LineFft<320, 40, 40, 8>, PACKED>(), variant<LineFft<384, 24, 24, 4, 4>, PACKED>(),
+    variant<LineFft<400, 20, 20, 20>, PACKED>(), variant<LineFft<512, 32, 32, 16>, PACKED>(),
+    variant<LineFft<768, 24, 24, 8, 4>, PACKED>(), variant<LineFft<1024, 32, 32, 32>, PACKED>(),
 };
 
+template <bool PACKED>
 const Variant *find(int n)
 {
-    for (const Variant &v : kVariants)
+    for (const Variant &v : kVariants<PACKED>)
         if (v.n == n)
             return &v;
     return nullptr;
+}
+
+bool packed(int nz) { return nz <= 2; }
+
+int items_of(int subgrids, int nz)
+{
+    return packed(nz) ? (subgrids * nz + kItemPlanes - 1) / kItemPlanes
+                      : subgrids * ((nz + kItemPlanes - 1) / kItemPlanes);
 }
 
 size_t item_bytes(int n) { return sizeof(float2) * (size_t)n * n * kItemPlanes; }
@@ -176,8 +188,8 @@ constexpr size_t kPassBytes = size_t(300) << 20;
 int choose_pass(const dg_predict_fft *p, int S, int most)
 {
     const auto cost = [&](int k) {
-        const double rows = ceil((double)k * p->groups * (p->n / kRowPair) / p->blocks_rows);
-        const double cols = ceil((double)k * p->groups * (p->n / kTileCols) / p->blocks_cols);
+        const double rows = ceil((double)items_of(k, p->nz) * (p->n / kRowPair) / p->blocks_rows);
+        const double cols = ceil((double)items_of(k, p->nz) * (p->n / kTileCols) / p->blocks_cols);
         return (2.8 * rows + 3.7 * cols) * p->n / 512 + 6.0;         // microseconds, roughly
     };
     int best = 1;
@@ -194,7 +206,7 @@ int choose_pass(const dg_predict_fft *p, int S, int most)
 
 }  // namespace
 
-bool dg_predict_fft_supported(int n, int nz) { return nz % kItemPlanes == 0 && find(n) != nullptr; }
+bool dg_predict_fft_supported(int n) { return find<true>(n) != nullptr; }
 
 void dg_predict_fft_destroy(dg_predict_fft *p)
 {
@@ -218,14 +230,12 @@ cudaError_t dg_predict_fft_create(dg_predict_fft **out, int n, int nz, int per_p
         return cudaErrorMemoryAllocation;
     p->n = n;
     p->nz = nz;
-    p->groups = nz / kItemPlanes;
-    p->v = find(n);
-    const size_t sub = item_bytes(n) * p->groups;
-    const size_t fit = kPassBytes / sub;
+    p->v = packed(nz) ? find<true>(n) : find<false>(n);
+    const size_t fit = packed(nz) ? kPassBytes / item_bytes(n) * (kItemPlanes / nz) : kPassBytes / (item_bytes(n) * items_of(1, nz));
     p->pass = fit < 1 ? 1 : (size_t)per_pass < fit ? per_pass : (int)fit;
     e = p->v->prepare(p, device, sm_count);
     if (e == cudaSuccess)
-        e = cudaMalloc((void **)&p->work, sub * p->pass);
+        e = cudaMalloc((void **)&p->work, item_bytes(n) * items_of(p->pass, nz));
     if (e == cudaSuccess)
         e = cudaMalloc((void **)&p->nm1, sizeof(float2) * (n / 2 + 1) * (n / 2 + 1));
     if (e != cudaSuccess) {
@@ -247,7 +257,7 @@ cudaError_t dg_predict_fft_execute(dg_predict_fft *p, cudaStream_t st, double th
     const int pass = choose_pass(p, n_subgrids, p->pass);
     for (int first = 0; first < n_subgrids && e == cudaSuccess; first += pass) {
         const int count = n_subgrids - first < pass ? n_subgrids - first : pass;
-        const PassItems items{first * p->groups, count * p->groups, p->groups};
+        const PassItems items{first, count, p->nz, items_of(count, p->nz), items_of(1, p->nz)};
         const int units = items.count * (p->n / kRowPair), tiles = items.count * (p->n / kTileCols);
         const RowsArgs ra{reinterpret_cast<const float2 *>(image), taper, w_planes, items, first == 0};
         e = p->v->rows(p, st, units < p->blocks_rows ? units : p->blocks_rows, ra);

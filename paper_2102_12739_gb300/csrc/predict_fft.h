@@ -6,8 +6,8 @@
 
 struct dg_predict_fft;
 
-// Whether images of n x n pixels with nz w-planes have a fused transform.
-bool dg_predict_fft_supported(int n, int nz);
+// Whether images of n x n pixels have a fused transform.
+bool dg_predict_fft_supported(int n);
 cudaError_t dg_predict_fft_create(dg_predict_fft **out, int n, int nz, int per_pass, int device);
 void dg_predict_fft_destroy(dg_predict_fft *p);
 cudaError_t dg_predict_fft_execute(dg_predict_fft *p, cudaStream_t st, double theta, const float *image,

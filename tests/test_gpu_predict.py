@@ -62,13 +62,14 @@ def test_small_stacks_every_cell(n, nz, theta, per_pass):
 
 
 @pytest.mark.parametrize("n,nz,S,per_pass", [
-    (64, 4, 5, 4), (96, 8, 3, 2), (128, 4, 3, 2), (192, 12, 2, 1), (256, 4, 3, 8), (320, 4, 2, 1), (384, 8, 2, 2),
+    (64, 4, 5, 4), (96, 8, 3, 2), (128, 4, 3, 2), (192, 12, 2, 1), (200, 4, 3, 2), (200, 3, 2, 2), (256, 4, 3, 8), (320, 4, 2, 1), (384, 8, 2, 2),
     (400, 4, 3, 2), (512, 4, 3, 1), (768, 4, 2, 2), (1024, 4, 1, 1),
-    (72, 4, 2, 2), (64, 6, 2, 2),               # no fused transform: the library's
+    (64, 1, 5, 4), (96, 3, 5, 3), (128, 6, 3, 2), (256, 2, 5, 5), (384, 5, 3, 3), (512, 1, 2, 2), (64, 3, 1, 1),
+    (72, 4, 2, 2), (72, 3, 2, 2),               # no fused transform: the library's
 ])
 def test_every_transform_size(n, nz, S, per_pass):
-    # each size of the fused transform: one and several plane groups, a ragged
-    # last pass, windows that wrap on both axes, a plane spacing that changes
+    # each size of the fused transform: one and several plane groups, groups of
+    # several subgrids' planes (one or two each), ragged last groups and passes, windows that wrap on both axes, a plane spacing that changes
     # between items, pixels outside the unit circle (theta 1.6)
     rng = np.random.default_rng(n + nz)
     img = (rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))).astype(np.complex64)
