@@ -22,11 +22,13 @@
 //
 // What bounds it is the L1 data path, a line or 128 bytes of shared memory
 // per cycle: a visibility's weights take two lines in and two reads out, its
-// share of M two to four reads.  When four lanes shared a visibility and read
+// share of M one to four reads.  When four lanes shared a visibility and read
 // the table themselves its weights took eight line accesses, and a step with
-// several runs one pass per run and eight visibilities: 166 us against 92 for
+// several runs one pass per run and eight visibilities: 166 us against 88 for
 // 2.5M visibilities on 24 subgrids' lines and arcs (123 with the weights loaded
-// by every lane itself, a line access per 32 bytes).
+// by every lane itself, a line access per 32 bytes), 298 against 289 for 16M on
+// 64 subgrids' lines (336 when every visibility's block was copied: its 4.1 GB
+// come from L2).
 #include "footprint.cuh"
 #include "pipeline.cuh"
 
@@ -46,9 +48,14 @@ struct alignas(16) MSlot {
 };
 
 struct alignas(128) WarpSmem {
-    float4 w[kBatch][kPieces];              // weight blocks of the step (piece q of row r at q ^ (r & 7))
+    float4 w[kBatch][kPieces];              // weight blocks of the step (piece q of row r at place(r, q))
     MSlot slot[kSlots];
+    int blk[kBatch];                        // which block each row of w holds
 };
+
+// Place of piece q of row r in the stage: the same piece of eight consecutive
+// rows lies in eight different bank groups.
+__device__ __forceinline__ int place(int r, int q) { return q ^ (r & 7); }
 
 // What the M builds of a warp need besides the footprint.
 struct BuildArgs {
@@ -84,6 +91,7 @@ struct Vis {
     int key;            // footprint start, -1: invalid or past the end of the step
     int fw;             // w row
     int blk;            // weight block fv * O + fu
+    int row;            // row of the stage that holds it
 };
 
 __device__ __forceinline__ Vis snap_step(const Batch &b, const Coords3 &c, const Geometry &g, DeviceStatus *status,
@@ -103,18 +111,37 @@ __device__ __forceinline__ Vis snap_step(const Batch &b, const Coords3 &c, const
     r.key = valid ? (vc.y0 * g.nx + vc.x0) * g.nz + vc.z0 : -1;
     r.fw = valid ? vc.fw : 0;
     r.blk = valid ? (vc.fv << g.log2_uv_os) + vc.fu : 0;
+    r.row = lane;
     return r;
 }
 
 // Starts the copies of a step's weight blocks (one cp.async group).
-__device__ __forceinline__ void copy_weights(WarpSmem &ws, const Vis &v, const float *__restrict__ g2, int lane)
+// Consecutive visibilities with one block share a row of the stage: on dense
+// lists the snapped offsets move slower than the visibilities.
+__device__ __forceinline__ void copy_weights(WarpSmem &ws, Vis &v, const float *__restrict__ g2, int lane)
 {
-    const int q = lane & (kPieces - 1);
+    const int before = __shfl_up_sync(kFull, v.blk, 1);
+    const bool head = lane == 0 || v.blk != before;
+    const unsigned heads = __ballot_sync(kFull, head);
+    const int rows = __popc(heads), q = lane & (kPieces - 1);
+    if (rows > kBatch / 2) {
+        v.row = lane;
 #pragma unroll
-    for (int i = 0; i < kBatch / 2; ++i) {
-        const int r = 2 * i + (lane >> 4);
-        const int blk = __shfl_sync(kFull, v.blk, r);
-        cp_async16(smem_u32(&ws.w[r][q ^ (r & 7)]), g2 + (size_t)blk * kBlock + 4 * q);
+        for (int i = 0; i < kBatch; i += 2) {
+            const int r = i + (lane >> 4);
+            const int blk = __shfl_sync(kFull, v.blk, r);
+            cp_async16(smem_u32(&ws.w[r][place(r, q)]), g2 + (size_t)blk * kBlock + 4 * q);
+        }
+    } else {
+        v.row = __popc(heads & (kFull >> (31 - lane))) - 1;
+        if (head)
+            ws.blk[v.row] = v.blk;
+        __syncwarp();
+        for (int i = 0; i < rows; i += 2) {
+            const int r = i + (lane >> 4);
+            if (r < rows)
+                cp_async16(smem_u32(&ws.w[r][place(r, q)]), g2 + (size_t)ws.blk[r] * kBlock + 4 * q);
+        }
     }
     cp_async_commit();
 }
@@ -133,10 +160,33 @@ __device__ __forceinline__ float combine(const float (&q)[4])
     return v + (e + (e0 + e1));
 }
 
+// Sum of row b of the footprint with row b of the weights in stage row `row`,
+// an FMA chain of (re, im) pairs.
+__device__ __forceinline__ float2 row_sum(const float4 (&m)[4], const WarpSmem &ws, int row, int b)
+{
+    const float4 w0 = ws.w[row][place(row, 2 * b)], w1 = ws.w[row][place(row, 2 * b + 1)];
+    float2 t = __fmul2_rn(make_float2(m[0].x, m[0].y), make_float2(w0.x, w0.x));
+    t = __ffma2_rn(make_float2(m[0].z, m[0].w), make_float2(w0.y, w0.y), t);
+    t = __ffma2_rn(make_float2(m[1].x, m[1].y), make_float2(w0.z, w0.z), t);
+    t = __ffma2_rn(make_float2(m[1].z, m[1].w), make_float2(w0.w, w0.w), t);
+    t = __ffma2_rn(make_float2(m[2].x, m[2].y), make_float2(w1.x, w1.x), t);
+    t = __ffma2_rn(make_float2(m[2].z, m[2].w), make_float2(w1.y, w1.y), t);
+    t = __ffma2_rn(make_float2(m[3].x, m[3].y), make_float2(w1.z, w1.z), t);
+    return __ffma2_rn(make_float2(m[3].z, m[3].w), make_float2(w1.w, w1.w), t);
+}
+
+__device__ __forceinline__ void load_row(float4 (&m)[4], const MSlot &slot, int b)
+{
+    const float4 *p = reinterpret_cast<const float4 *>(&slot.m[b][0]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        m[k] = p[k];
+}
+
 // The lane's visibility from the footprint in `slot`: quarter j is the sum of
-// rows 2j and 2j + 1, a row an FMA chain of (re, im) pairs.
+// rows 2j and 2j + 1.
 template <bool COMP>
-__device__ __forceinline__ float2 sum_lane(const MSlot &slot, const WarpSmem &ws, int lane)
+__device__ __forceinline__ float2 sum_lane(const MSlot &slot, const WarpSmem &ws, int row)
 {
     float qx[4], qy[4];
 #pragma unroll
@@ -144,22 +194,51 @@ __device__ __forceinline__ float2 sum_lane(const MSlot &slot, const WarpSmem &ws
         float2 R[2];
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            const int b = 2 * j + i;
-            const float4 *m = reinterpret_cast<const float4 *>(&slot.m[b][0]);
-            const float4 m0 = m[0], m1 = m[1], m2 = m[2], m3 = m[3];
-            const float4 w0 = ws.w[lane][(2 * b) ^ (lane & 7)], w1 = ws.w[lane][(2 * b + 1) ^ (lane & 7)];
-            float2 t = __fmul2_rn(make_float2(m0.x, m0.y), make_float2(w0.x, w0.x));
-            t = __ffma2_rn(make_float2(m0.z, m0.w), make_float2(w0.y, w0.y), t);
-            t = __ffma2_rn(make_float2(m1.x, m1.y), make_float2(w0.z, w0.z), t);
-            t = __ffma2_rn(make_float2(m1.z, m1.w), make_float2(w0.w, w0.w), t);
-            t = __ffma2_rn(make_float2(m2.x, m2.y), make_float2(w1.x, w1.x), t);
-            t = __ffma2_rn(make_float2(m2.z, m2.w), make_float2(w1.y, w1.y), t);
-            t = __ffma2_rn(make_float2(m3.x, m3.y), make_float2(w1.z, w1.z), t);
-            R[i] = __ffma2_rn(make_float2(m3.z, m3.w), make_float2(w1.w, w1.w), t);
+            float4 m[4];
+            load_row(m, slot, 2 * j + i);
+            R[i] = row_sum(m, ws, row, 2 * j + i);
         }
         const float2 q = __fadd2_rn(R[0], R[1]);
         qx[j] = q.x;
         qy[j] = q.y;
+    }
+    return make_float2(combine<COMP>(qx), combine<COMP>(qy));
+}
+
+// The same when the whole step is on one footprint: lanes l and l + 16 take
+// four rows each for both of their visibilities, which halves the reads of the
+// footprint, and exchange two quarters.  (Neighbouring lanes, so that both
+// rows are read within eight lanes, gained nothing: 318 us for 16M
+// visibilities on 64 subgrids' lines, 314 without sharing, 289 like this.)
+template <bool COMP>
+__device__ __forceinline__ float2 sum_pair(const MSlot &slot, const WarpSmem &ws, int row, int lane)
+{
+    const int h = lane >> 4, other = __shfl_xor_sync(kFull, row, 16);
+    const int ra = h ? other : row, rb = h ? row : other;       // stage rows of the lower and the upper lane
+    float2 qa[2], qb[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        float2 A[2], B[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int b = 4 * h + 2 * j + i;
+            float4 m[4];
+            load_row(m, slot, b);
+            A[i] = row_sum(m, ws, ra, b);
+            B[i] = row_sum(m, ws, rb, b);
+        }
+        qa[j] = __fadd2_rn(A[0], A[1]);
+        qb[j] = __fadd2_rn(B[0], B[1]);
+    }
+    float qx[4], qy[4];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const float2 give = h ? qa[j] : qb[j], keep = h ? qb[j] : qa[j];
+        const float2 got = make_float2(__shfl_xor_sync(kFull, give.x, 16), __shfl_xor_sync(kFull, give.y, 16));
+        qx[j] = h ? got.x : keep.x;
+        qy[j] = h ? got.y : keep.y;
+        qx[j + 2] = h ? keep.x : got.x;
+        qy[j + 2] = h ? keep.y : got.y;
     }
     return make_float2(combine<COMP>(qx), combine<COMP>(qy));
 }
@@ -221,7 +300,7 @@ __device__ __forceinline__ float2 sum_runs(MCache &mc, WarpSmem &ws, int64_t bas
         }
         __syncwarp();
         const bool mine = v.key >= 0 && run >= first && run < first + n;
-        const float2 x = sum_lane<COMP>(ws.slot[(start + (mine ? run - first : 0)) & (kSlots - 1)], ws, lane);
+        const float2 x = sum_lane<COMP>(ws.slot[(start + (mine ? run - first : 0)) & (kSlots - 1)], ws, v.row);
         if (mine)
             V = x;
     }
@@ -257,7 +336,7 @@ degrid_2d_kernel(const Geometry g, const void *__restrict__ subgrids, const floa
     int64_t base = 0;
     float sc = 1.f;
     while (true) {
-        const Vis vB = snap_step(bB, c, g, status, lane);
+        Vis vB = snap_step(bB, c, g, status, lane);
         const Batch bC = claimer.advance(bB);
         c = load_uvw(uvw, bC, lane);
 
@@ -272,7 +351,7 @@ degrid_2d_kernel(const Geometry g, const void *__restrict__ subgrids, const floa
         __syncwarp();                   // every lane's copies of the weights
         float2 V;
         if (__all_sync(kFull, vA.key == mc.key && vA.fw == mc.fw))
-            V = sum_lane<COMP>(ws.slot[mc.slot], ws, lane);     // the step continues the cached run
+            V = sum_pair<COMP>(ws.slot[mc.slot], ws, vA.row, lane);   // the step continues the cached run
         else
             V = sum_runs<DT, COMP>(mc, ws, base, vA, g, A);
         if (DT != DG_C64)
