@@ -45,10 +45,11 @@ FLOP_PER_VIS = 1024          # 256 footprint points x complex*real FMA (2 FMA = 
 # all proportional to the visibilities).  Valid only for the kernel sources it was taken
 # on: the bench reports null traffic once they change.
 TRAFFIC_KERNEL_SOURCES = ("paper_2102_12739_gb300/csrc/degrid.cu",
+                          "paper_2102_12739_gb300/csrc/footprint.cuh",
                           "paper_2102_12739_gb300/csrc/pipeline.cuh",
                           "paper_2102_12739_gb300/csrc/internal.cuh")
-TRAFFIC_SHA = "a15f6785f22862b7"
-TRAFFIC_BYTES_PER_VIS = (98.424320e6 + 11.519232e6) / 4_000_000
+TRAFFIC_SHA = "5f84fad245c2e04d"
+TRAFFIC_BYTES_PER_VIS = (98.423808e6 + 11.627776e6) / 4_000_000
 FP32_LANES_PER_SM = 128
 L2_FLUSH_BYTES = 256 << 20
 # (chunk, warps per CTA, CTAs per SM, direct-arm threshold) tried on the headline workload
@@ -441,7 +442,8 @@ def scatter_section(torch, dg, synth, dev, flush, steps, l2_gbs):
                    "tuning": tuned["tuning"]}
         del codes, scale
     # gridding (the adjoint) of the same coverage: the run-accumulating kernel
-    # (atomic adds at every run end) and the tensor reduce-add kernel
+    # (atomic adds at every run end) and the gather setting's (tensor
+    # reduce-adds, here of whole tiles, which can pass the bound below)
     y = torch.from_numpy(synth.adjoint_vis(w.n_vis)).to(dev)
     grid_out = torch.empty((w.n_subgrids,) + w.shape, dtype=torch.complex64, device=dev)
     gridding = {}
@@ -458,8 +460,8 @@ def scatter_section(torch, dg, synth, dev, flush, steps, l2_gbs):
         kms = k_ms[len(k_ms) // 2]
         gridding["tensor reduce-add" if gather else "run accumulation + atomics"] = {
             "kernel_ms": kms, "value": w.n_vis / (kms * 1e-3), "unit": "gridded visibilities/s"}
-    # the reduce-add kernel's bound: every visibility adds its 2 KB footprint
-    # tile, at the measured rate of the copy engines' tensor reduce-adds
+    # the bound of adding every visibility's 2 KB footprint by itself, at the
+    # measured rate of the copy engines' tensor reduce-adds
     red_gbs = dg.measure_l2_reduce_bw(dev.index)
     red = gridding["tensor reduce-add"]
     red["reduce_bound_ms"] = w.n_vis * 2048 / (red_gbs * 1e9) * 1e3
@@ -516,8 +518,8 @@ def latency_section(torch, dg, synth, dev, steps):
             "timing": "call_us: GPU time of one call with the queue filled ahead (events on the "
                       "stream, medians); call_us_host_paced: calls issued back to back as the host "
                       "enqueues them, so the host's own enqueue time can show",
-            "call_includes": "one scheduling launch (offset validation, chunk scan and chunk "
-                             "table) and the degridding kernel"}
+            "call_includes": "the degridding kernel, which takes its pieces of the lists from the "
+                             "offsets itself (no scheduling launch for a call this small)"}
 
 
 def table2d_section(torch, dg, synth, dev, flush, steps, sub, sub_np, uvw, offs, w):
@@ -610,8 +612,8 @@ def predict_section(torch, dg, synth, dev, flush, steps, hbm_gbs, plan=None, uvw
                     "100 wavelengths apart covering -12800..12800 wavelengths",
         "value": S / (ms * 1e-3), "unit": "subgrids/s", "ms_per_call": ms, "steps": steps,
         "subgrids_per_pass": per_pass,
-        "kernels": "screen_kernel (tapered image x w-phase screens), batched 512x512 C2C FFT (cuFFT), "
-                   "window_kernel (cell window, sign, [y][x][c] interleave)",
+        "kernels": "rows_kernel (tapered image x w-phase screens, row transforms), columns_kernel "
+                   "(column transforms, cell window, [y][x][c] interleave)",
         "hbm_bytes_compulsory": out_bytes + in_bytes, "hbm_bound_ms": bound_ms,
         "hbm_frac": bound_ms / ms,
         "rel_l2_vs_oracle": err[0], "max_abs_vs_oracle": err[1], "error_sample": "all"})

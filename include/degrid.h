@@ -196,9 +196,9 @@ dg_status degrid_plan_get_compensated(degrid_plan_t plan, int *enabled);
 /*
  * Summing arm for short runs (the paper's per-visibility kernels D1/D2 next
  * to the footprint-reuse path, Section "Implementation").  degrid_execute
- * works on halves of 32 consecutive visibilities.  A half whose visibilities
- * share one footprint and w row reuses the cached footprint sum M; any other
- * half with at least min_runs runs of equal (footprint, w row) is summed
+ * of a plan with the arm enabled works on halves of 32 consecutive
+ * visibilities.  A half whose visibilities share one footprint and w row
+ * reuses the cached footprint sum M; any other half with at least min_runs runs of equal (footprint, w row) is summed
  * directly, every visibility from its own 8 x 8 x 4 footprint (no cache
  * rebuilds), and halves with fewer runs rebuild M per run.  Both arms do the
  * same arithmetic in the same order, so the results are bitwise identical;
@@ -206,7 +206,7 @@ dg_status degrid_plan_get_compensated(degrid_plan_t plan, int *enabled);
  * overlap but change often (w rows changing every few visibilities) and
  * loses on footprints scattered over the subgrid.  min_runs: 1 ..
  * DG_DIRECT_RUNS_NEVER (33: never, the default; a plan with the arm enabled
- * launches another instance of the kernel).  DG_DIRECT_RUNS_SHORT is the
+ * launches another kernel, which has four lanes share a visibility).  DG_DIRECT_RUNS_SHORT is the
  * setting the autotuner tries.  Returns DG_OK or DG_ERR_ARG.
  */
 #define DG_DIRECT_RUNS_NEVER 33
@@ -218,21 +218,35 @@ dg_status degrid_plan_get_direct_runs(degrid_plan_t plan, int *min_runs);
 /*
  * Gather arm for sparse coverage (lists whose consecutive visibilities
  * rarely share a footprint: the short-list regime of the paper's kernels
- * D2/D4, Section "Results").  With enabled = 1, degrid_execute streams every
- * visibility's own 8 x 8 x 4 footprint into shared memory with asynchronous
- * copies, several footprints in flight per warp, instead of caching the
- * footprint sum M per run; a separate kernel with one CTA per SM (12 warps
- * for complex64, 22 for FP16/BF16), so the warps_per_block and
- * blocks_per_sm of the tuning do not apply to it (the chunk size does).
- * Same arithmetic in the same order as the footprint-cache path: results
+ * D2/D4, Section "Results").  With enabled = 1, degrid_execute does not
+ * cache the footprint sum M per run, but
+ *  - calls with many visibilities (100,000 and 14 for every 32 x 32
+ *    footprint starts of the stack; subgrids of at least 48 x 48 with at most
+ *    4096 such tiles, at most 65,535 subgrids and 2^26 visibilities) sort
+ *    them by tile and keep each tile's part of the subgrid in shared memory
+ *    while its visibilities are summed.  The workspace (16 bytes per
+ *    visibility and a little) belongs to the plan and grows with the largest
+ *    call; a call that cannot grow it (inside a stream capture, no memory)
+ *    goes the next way;
+ *  - others stream every visibility's own 8 x 8 x 4 footprint into shared
+ *    memory with asynchronous copies, several footprints in flight per warp:
+ *    a separate kernel with one CTA per SM (12 warps for complex64, 22 for
+ *    FP16/BF16);
+ *  - calls with too few visibilities for either (64 per resident warp, at
+ *    most 256 subgrids) run as without the setting.
+ * The warps_per_block and blocks_per_sm of the tuning do not apply to the
+ * first two (the chunk size does to the second).  Same arithmetic in the same order as the footprint-cache path: results
  * are bitwise identical; the compensated setting applies.  Only the speed
  * differs: it wins when footprints are scattered and loses on dense lists,
  * where one cached M serves hundreds of visibilities.  The setting also
  * switches grid_adjoint_execute (output stack 16-byte aligned) to its
- * counterpart for scattered coverage: each visibility's 8 x 8 x 4
- * contribution is written to shared memory and added to the stack by one
- * tensor reduce-add of the copy engine, instead of the run accumulation
- * with atomic adds at run ends (FP32 additions in another order: the last
+ * counterparts for scattered coverage, instead of the run accumulation with
+ * atomic adds at run ends: calls with many visibilities (50,000 and 11 for
+ * every 16 x 16 footprint starts, the other limits as above) add them tile by
+ * tile in shared memory and each tile to the stack; others write each
+ * visibility's 8 x 8 x 4 contribution to shared memory and add it to the stack
+ * by one tensor reduce-add of the copy engine; small calls (32 visibilities
+ * per resident warp) run as without the setting (FP32 additions in another order: the last
  * bits differ).  Needs nz = 4 and a separable G_uv table: enabling it on another
  * plan returns DG_ERR_UNSUPPORTED.  Calls whose stack has more than
  * 2^31 - 1 rows in all (n_subgrids * ny) take the footprint-cache kernels
@@ -251,7 +265,8 @@ dg_status degrid_plan_get_tuning(degrid_plan_t plan, int *chunk, int *warps_per_
  * with n_slots > 0 creates n_slots CUDA event pairs; from then on every
  * degrid_execute / grid_adjoint_execute records one pair on its stream around
  * its main (persistent) kernel only, excluding the small scheduling
- * kernels, cycling through the slots.  n_slots = 0 disables timing and frees
+ * kernels (calls that go by tiles, see degrid_plan_set_gather: the sort
+ * included), cycling through the slots.  n_slots = 0 disables timing and frees
  * the events.  Disable timing before capturing calls into a CUDA graph.
  *
  * degrid_plan_kernel_times_ms synchronises on the newest pair and writes the
@@ -422,8 +437,8 @@ dg_status degrid_pack_subgrids(void *stream, dg_dtype dtype, int n_subgrids, int
  * Read and clear the device-side status of the plan: synchronises `stream`,
  * stores the number of invalid visibilities seen since the last call in
  * *n_invalid (may be NULL) and returns DG_ERR_TIMEOUT if a bounded wait of
- * a kernel gave up (the gather kernel's waits on its copies; the results of
- * that call are incomplete), else DG_ERR_BOUNDS if the library was built
+ * a kernel gave up (the waits of the gather and tile kernels on their copies;
+ * the results of that call are incomplete), else DG_ERR_BOUNDS if the library was built
  * with DEGRID_BOUNDS_CHECK and an index the coordinate step produced fell
  * outside its buffer (that visibility was skipped), else DG_ERR_OFFSETS if a
  * call saw malformed vis_offsets, else DG_OK (or DG_ERR_CUDA).

@@ -199,9 +199,10 @@ class DegridPlan:
         return v.value
 
     def set_gather(self, enabled: bool = True) -> None:
-        """Sum through the gather kernel (every footprint streamed into shared
-        memory; for scattered coverage).  Results are bitwise the same as the
-        footprint-cache path.  Needs nz = 4 and a separable G_uv table."""
+        """For scattered coverage: large calls sorted by tile, others through
+        the gather kernel (every footprint streamed into shared memory); grid()
+        likewise.  Sums are bitwise the same as the footprint-cache path's.
+        Needs nz = 4 and a separable G_uv table."""
         check(load().degrid_plan_set_gather(self.handle, 1 if enabled else 0),
               "degrid_plan_set_gather")
 

@@ -19,7 +19,7 @@
 // Measured on 64 subgrids of 512 x 512 x 4: 653 -> 355 us a call (21 of
 // 384 x 384 x 4: 239 -> 92 us); with 1, 2, 3, 5 and 7 planes 287 -> 165, 427
 // -> 262, 576 -> 385, 917 -> 831 and 1240 -> 997 us; 64 of 200 x 200 x 3 148
-// -> 86 us.  Of each 32 subgrids the row kernel takes 97
+// -> 88 us.  Of each 32 subgrids the row kernel takes 97
 // us at 44% of the issue slots (51 instructions per point, 31 of them FP32),
 // the column kernel 87 us at 6.2 TB/s of DRAM traffic.
 #pragma once
