@@ -15,7 +15,7 @@
 // visibility, 32 accesses of 128 bytes at one per cycle and SM, where the
 // scatter kernel's reduce-adds of single footprints ran at the 6.5 TB/s the
 // copy engines add into L2.  2M visibilities scattered over 16 subgrids, with
-// the sort and the zeros: 698 -> 395 us.  Tiles of 8 x 8 (28 warps), 8 x 16
+// the sort and the zeros: 698 -> 391 us.  Tiles of 8 x 8 (28 warps), 8 x 16
 // and 16 x 8 (20) measured 458, 407 and 406: the adds of the regions grow.
 //
 // Requirements (checked by the host): as the scatter kernel.
