@@ -5,7 +5,9 @@
 // tensor copy, and its warps sum the item's visibilities four at a time: lane
 // 8v + b takes row b of visibility v,
 //     R_b = sum_a g_u[a] sum_c g_w[c] s[b][a][c],
-// and the eight lanes of a visibility combine as in the gather kernel.  Every
+// and the eight lanes of a visibility combine as in the gather kernel, two
+// steps' visibilities at a time (the even lanes end with one, the odd lanes
+// with the other: half the shuffles).  Every
 // operation and its order match the gather and footprint-cache kernels, so
 // all three agree bit for bit.  A region row is 16 bytes more than a multiple
 // of 128, so the eight rows of a footprint start in eight different bank
@@ -15,9 +17,10 @@
 // What bounds it: 16 reads of 128 bytes from shared memory per visibility
 // in complex64 (8 in FP16/BF16) at one per cycle and SM, where the gather
 // kernel's 2.3 KB per visibility came from L2.  With the rows of the tables,
-// the records and the shuffles it is 25 cycles per visibility, 82% of the
+// the records and the shuffles it is 24 cycles per visibility, 80% of the
 // data path's.  4M visibilities scattered over 16 subgrids, with the sort:
-// 565 -> 391 us in complex64; 1.2M over 13 in FP16, compensated: 170 -> 129.
+// 565 -> 380 us in complex64; 1.2M over 13 in FP16, compensated: 170 -> 124
+// (391 and 129 with the shuffles of every visibility by itself).
 //
 // Requirements (checked by the host): as the gather kernel.
 #include "bins.cuh"
@@ -99,8 +102,9 @@ __device__ __forceinline__ void column(const unsigned char *row, int a, float2 (
     }
 }
 
-template <int DT, bool COMP>
-__device__ __forceinline__ float2 sum_visibility(const unsigned char *region, const LaneVis &v, const float4 &gw, int b)
+// This lane's row of the visibility: R_b.
+template <int DT>
+__device__ __forceinline__ float2 sum_row(const unsigned char *region, const LaneVis &v, const float4 &gw, int b)
 {
     const int lx = v.r.ux >> kBinRowBits, ly = v.r.vy >> kBinRowBits;
     const unsigned char *row = region + (ly + b) * RegionShape<DT>::kPitch + lx * (kW * Storage<DT>::kBytes);
@@ -115,10 +119,22 @@ __device__ __forceinline__ float2 sum_visibility(const unsigned char *region, co
         m = __ffma2_rn(s[3], make_float2(gw.w, gw.w), m);
         R = a == 0 ? __fmul2_rn(m, make_float2(v.gu[0], v.gu[0])) : __ffma2_rn(m, make_float2(v.gu[a], v.gu[a]), R);
     }
+    return R;
+}
+
+// The eight lanes of a visibility each have a row of it, RA of the group's
+// visibility A and RB of its B: the even lanes end with A's sum, the odd ones
+// with B's.  `gv`: the g_v pair of this lane's quarter, of A or B.  (Reducing
+// one visibility at a time takes twice the shuffles.)
+template <bool COMP>
+__device__ __forceinline__ float2 sum_rows(const float2 &RA, const float2 &RB, const float2 &gv, int b)
+{
     // quarter j = b >> 1: g_v[2j + 1] R_{2j + 1} + g_v[2j] R_{2j}
-    const float2 Rn = make_float2(__shfl_xor_sync(kFull, R.x, 1), __shfl_xor_sync(kFull, R.y, 1));
-    const float2 Re = (b & 1) ? Rn : R, Ro = (b & 1) ? R : Rn;
-    const float2 Q = __ffma2_rn(Ro, make_float2(v.gv.y, v.gv.y), __fmul2_rn(Re, make_float2(v.gv.x, v.gv.x)));
+    const bool odd = b & 1;
+    const float2 give = odd ? RA : RB, own = odd ? RB : RA;
+    const float2 got = make_float2(__shfl_xor_sync(kFull, give.x, 1), __shfl_xor_sync(kFull, give.y, 1));
+    const float2 Re = odd ? got : own, Ro = odd ? own : got;
+    const float2 Q = __ffma2_rn(Ro, make_float2(gv.y, gv.y), __fmul2_rn(Re, make_float2(gv.x, gv.x)));
     // (Q_j + Q_{j^2}) + (Q_{j^1} + Q_{j^3})
     float2 V;
     if (COMP) {
@@ -190,18 +206,33 @@ tiled_degrid_kernel(const Geometry g, const __grid_constant__ CUtensorMap map, c
             break;
         }
         parity ^= 1;
-        for (int at = at0; at - v < it.n; at += kStep) {
+        // Sum this lane's row of the step at `at` and move on to the next.
+        const auto step = [&](int at) {
             LaneVis nv;
             nv.r = next;
             next = load_record(recs, at + 2 * kStep, at + 2 * kStep < it.n);
             load_rows(nv, guv, b);
             const float4 gw = wtab ? wtab[cur.r.fw] : __ldg(reinterpret_cast<const float4 *>(gwt) + cur.r.fw);
-            float2 V = sum_visibility<DT, COMP>(region, cur, gw, b);
+            const float2 R = sum_row<DT>(region, cur, gw, b);
+            cur = nv;
+            return R;
+        };
+        for (int at = at0; at - v < it.n; at += 2 * kStep) {
+            float2 gv = cur.gv;
+            unsigned index = cur.r.index;
+            const float2 RA = step(at);
+            if (b & 1) {
+                gv = cur.gv;
+                index = cur.r.index;
+            }
+            float2 RB = make_float2(0.f, 0.f);
+            if (at + kStep - v < it.n)      // the same in the whole warp
+                RB = step(at + kStep);
+            float2 V = sum_rows<COMP>(RA, RB, gv, b);
             if (DT != DG_C64)
                 V = __fmul2_rn(V, make_float2(sc, sc));
-            if (b == 0 && at < it.n)
-                vis_out[cur.r.index] = V;
-            cur = nv;
+            if (b < 2 && at + b * kStep < it.n)
+                vis_out[index] = V;
         }
     }
 }
