@@ -204,7 +204,7 @@ bool tma_rows_fit(const degrid_plan *p, int n_subgrids)
 // and the workspace fits (or can grow now).
 bool tiled(degrid_plan *p, cudaStream_t st, dg::TileShape shape, int n_subgrids, int64_t n_vis)
 {
-    return p->gather && dg_bins_worth(p, shape, n_subgrids, n_vis) && dg_bins_reserve(p, st, shape, n_subgrids, n_vis);
+    return p->gather && dg_bins_worth(p, shape, n_subgrids, n_vis) && dg_bins_reserve(p, st, n_subgrids, n_vis);
 }
 
 // The pieces of a call too small to need a chunk table: one step of at most

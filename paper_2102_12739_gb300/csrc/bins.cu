@@ -229,7 +229,7 @@ bool dg_bins_worth(const degrid_plan *p, dg::TileShape shape, int n_subgrids, lo
            p->geo.nx >= 48 && p->geo.ny >= 48;      // a region fits the subgrid
 }
 
-bool dg_bins_reserve(degrid_plan *p, cudaStream_t st, dg::TileShape shape, int n_subgrids, long long n_vis)
+bool dg_bins_reserve(degrid_plan *p, cudaStream_t st, int n_subgrids, long long n_vis)
 {
     if (!p->bins) {
         p->bins = new (std::nothrow) dg_bins();
@@ -237,7 +237,9 @@ bool dg_bins_reserve(degrid_plan *p, cudaStream_t st, dg::TileShape shape, int n
             return false;
     }
     dg_bins *b = p->bins;
-    const long long tiles = tiles_of(p, shape, n_subgrids), items = items_of(n_vis, tiles);
+    // for calls in both directions: growing the workspace costs a synchronisation
+    const long long td = tiles_of(p, kDegridTile, n_subgrids), tg = tiles_of(p, kGridTile, n_subgrids);
+    const long long tiles = td > tg ? td : tg, items = items_of(n_vis, tiles);
     if (n_vis <= b->cap_records && tiles <= b->cap_tiles && items <= b->cap_items)
         return true;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;

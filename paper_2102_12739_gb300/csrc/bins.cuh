@@ -73,7 +73,7 @@ struct dg_bins {
 bool dg_bins_worth(const degrid_plan *p, dg::TileShape shape, int n_subgrids, long long n_vis);
 // Grows the workspace; false when it is too small and cannot grow now (the
 // stream is capturing, or no memory is left).
-bool dg_bins_reserve(degrid_plan *p, cudaStream_t st, dg::TileShape shape, int n_subgrids, long long n_vis);
+bool dg_bins_reserve(degrid_plan *p, cudaStream_t st, int n_subgrids, long long n_vis);
 // Sorts the call's visibilities.  Invalid ones are counted and, with vis_out,
 // get their zero; malformed offsets are flagged.
 cudaError_t dg_bins_sort(degrid_plan *p, cudaStream_t st, dg::TileShape shape, int n_subgrids,
