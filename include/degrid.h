@@ -232,7 +232,7 @@ dg_status degrid_plan_get_direct_runs(degrid_plan_t plan, int *min_runs);
  *    memory with asynchronous copies, several footprints in flight per warp:
  *    a separate kernel with one CTA per SM (12 warps for complex64, 22 for
  *    FP16/BF16);
- *  - calls with too few visibilities for either (64 per resident warp, at
+ *  - calls with too few visibilities for either (32 per resident warp, at
  *    most 256 subgrids) run as without the setting.
  * The warps_per_block and blocks_per_sm of the tuning do not apply to the
  * first two (the chunk size does to the second).  Same arithmetic in the same order as the footprint-cache path: results

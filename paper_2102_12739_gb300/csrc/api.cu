@@ -233,30 +233,39 @@ constexpr int kDegridPieceLeast = 16;
 // 20,000 visibilities of lines and arcs on one subgrid: an error of 2.2e-7
 // against 1.5e-7 to FP64).  So a piece is what a chunk of such a call is.
 // With the gather setting the scatter kernel would add every visibility by
-// itself, so short pieces lose nothing (8 lists of 125: 21 us in pieces of 8,
-// 50 of 64).
+// itself, so short pieces lose nothing (8 lists of 125: 23 us in pieces of 8,
+// 42 of 64).
 int grid_piece_least(const degrid_plan *p) { return p->gather ? 8 : kPieceMost; }
 
-// The most visibilities per warp.  Scattered ones (the gather setting) are
-// gridded faster by the scatter kernel from about 80,000 on; up to the limit
-// they are degridded faster this way than by the gather kernel (20,000 on one
-// subgrid: 15 us against 40).
-int grid_piece_most(const degrid_plan *p) { return p->gather ? kPieceMost / 2 : kPieceMost; }
+// The most visibilities per warp.  Up to about 80,000 scattered ones (the
+// gather setting) are faster this way than by the gather and scatter kernels
+// (20,000 on one subgrid: degridding 40 -> 15 us, gridding 79 -> 20), more are
+// not (100,000 on 64 uneven lists: degridding 58 us against 54).
+int piece_most(const degrid_plan *p) { return p->gather ? kPieceMost / 2 : kPieceMost; }
+
+int piece_blocks_per_sm(const degrid_plan *p, int max_per_sm)
+{
+    return p->blocks_per_sm > 0 && p->blocks_per_sm < max_per_sm ? p->blocks_per_sm : max_per_sm;
+}
 
 dg::Pieces pieces_of(const degrid_plan *p, const int64_t *vis_offsets, int n_subgrids, int64_t n_vis, int max_per_sm,
                      int least, int most)
 {
-    const int per_sm = p->blocks_per_sm > 0 && p->blocks_per_sm < max_per_sm ? p->blocks_per_sm : max_per_sm;
-    const int64_t warps = (int64_t)p->sm_count * per_sm * p->warps_per_block;
+    const int64_t warps = (int64_t)p->sm_count * piece_blocks_per_sm(p, max_per_sm) * p->warps_per_block;
     const bool small = n_subgrids <= kPieceLists && n_vis <= warps * most;
     const int64_t share = (n_vis + warps - 1) / warps;
     return dg::Pieces{vis_offsets, n_subgrids, small ? (int)(share > least ? share : least) : 0, n_vis};
 }
 
-int piece_blocks(const degrid_plan *p, const dg::Pieces &pieces)
+// The resident CTAs, but no more than there are pieces: these go to the CTAs
+// in turn, so that few pieces spread over all SMs (gridding 60,000
+// visibilities of 8 uneven lists of lines and arcs: 54 us with neighbouring
+// pieces in one CTA, 42 like this, 54 with a chunk table).
+int piece_blocks(const degrid_plan *p, const dg::Pieces &pieces, int max_per_sm)
 {
-    const int64_t per_block = (int64_t)pieces.per_warp * p->warps_per_block;
-    return (int)((pieces.n_vis + per_block - 1) / per_block);
+    const int64_t n = (pieces.n_vis + pieces.per_warp - 1) / pieces.per_warp;
+    const int64_t blocks = (int64_t)p->sm_count * piece_blocks_per_sm(p, max_per_sm);
+    return (int)(blocks < n ? blocks : n);
 }
 
 // Persistent grid: the resident CTAs of every SM, but no more CTAs than
@@ -647,7 +656,7 @@ dg_status degrid_execute(degrid_plan_t p, void *stream, int n_subgrids, const vo
     dg::Pieces pieces{};
     if (dg_degrid_takes_pieces(p) && !(kKeepGather && p->gather))
         pieces = pieces_of(p, vis_offsets, n_subgrids, n_vis, p->max_blocks_degrid, kDegridPieceLeast,
-                           kPieceMost);
+                           piece_most(p));
     const bool gather = p->gather && pieces.per_warp == 0 && tma_rows_fit(p, n_subgrids);
     cudaError_t e = cudaSuccess;
     if (pieces.per_warp == 0)
@@ -664,7 +673,7 @@ dg_status degrid_execute(degrid_plan_t p, void *stream, int n_subgrids, const vo
         return from_cuda(e);
     }
     const int blocks = pieces.per_warp > 0
-                           ? piece_blocks(p, pieces)
+                           ? piece_blocks(p, pieces, p->max_blocks_degrid)
                            : grid_blocks(p, n_subgrids, n_vis, chunk, p->max_blocks_degrid, p->warps_per_block);
     KernelTimer timer(p, s);
     e = dg_launch_degrid(p, s, subgrids, subgrid_scale, uvw, pieces, vis_out, blocks);
@@ -703,7 +712,7 @@ dg_status grid_adjoint_execute(degrid_plan_t p, void *stream, int n_subgrids, co
     if (p->max_blocks_adjoint == 0)
         p->max_blocks_adjoint = dg_max_blocks_per_sm_adjoint(p);
     const dg::Pieces pieces = pieces_of(p, vis_offsets, n_subgrids, n_vis, p->max_blocks_adjoint,
-                                        grid_piece_least(p), grid_piece_most(p));
+                                        grid_piece_least(p), piece_most(p));
     if (pieces.per_warp == 0 && aligned(sub_out, 16) && tiled(p, s, kGridTile, n_subgrids, n_vis)) {
         KernelTimer timer(p, s);
         dg::Bins bins;
@@ -729,7 +738,7 @@ dg_status grid_adjoint_execute(degrid_plan_t p, void *stream, int n_subgrids, co
         return from_cuda(e);
     }
     const int blocks = pieces.per_warp > 0
-                           ? piece_blocks(p, pieces)
+                           ? piece_blocks(p, pieces, p->max_blocks_adjoint)
                            : grid_blocks(p, n_subgrids, n_vis, chunk, p->max_blocks_adjoint, p->warps_per_block);
     KernelTimer timer(p, s);
     e = dg_launch_adjoint(p, s, uvw, pieces, vis_in, sub_out, blocks);

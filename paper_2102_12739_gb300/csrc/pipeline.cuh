@@ -159,7 +159,7 @@ struct PieceClaimerT {
 
     __device__ PieceClaimerT(const Pieces &p, int lane_) : pieces(p), lane(lane_), lo(0), hi(0), next(0), todo(0)
     {
-        const long long k = (long long)blockIdx.x * (blockDim.x / kWarp) + threadIdx.x / kWarp;
+        const long long k = (long long)(threadIdx.x / kWarp) * gridDim.x + blockIdx.x;
         first = k * p.per_warp;
         last = min(first + p.per_warp, (long long)p.n_vis);
     }
