@@ -207,14 +207,23 @@ bool tiled(degrid_plan *p, cudaStream_t st, dg::TileShape shape, int n_subgrids,
     return p->gather && dg_bins_worth(p, shape, n_subgrids, n_vis) && dg_bins_reserve(p, st, n_subgrids, n_vis);
 }
 
-// The pieces of a call too small to need a chunk table: one step of at most
-// `most` visibilities for every resident warp, which saves the scheduling
+// The pieces of a call too small to need a chunk table: steps of at most
+// `most` visibilities, one for every resident warp, which saves the scheduling
 // kernel's launch and run (20,000 visibilities on a line: 12.3 -> 4.6 us of
 // GPU time).  If there are not enough visibilities for all warps, a piece has
 // `least` of them.  Few enough lists for every warp to look at all of them.
 // per_warp 0: not such a call.
 constexpr int kPieceMost = 64;          // one step
 constexpr int kPieceLists = 256;
+
+// With few lists a call may have several pieces per warp, a grid of warps
+// apart, up to where calls get chunks of more than one step: degridding
+// 300,000 visibilities of one line 24 -> 15 us, of 8 uneven lists 30 -> 27,
+// scattered over one subgrid 138 -> 97; gridding 31 -> 23, 42 -> 40, 224 ->
+// 164.  With more uneven lists the claims of the chunk table balance better
+// (450,000 visibilities: 32 lists 73 us against 87, 200 lists 73 against 91).
+constexpr int kPieceRounds = 4;
+constexpr int kRoundLists = 16;
 
 // The library variant that tests the gather kernel's bounded wait keeps small
 // calls of plans with the gather setting on that kernel.
@@ -252,8 +261,9 @@ dg::Pieces pieces_of(const degrid_plan *p, const int64_t *vis_offsets, int n_sub
                      int least, int most)
 {
     const int64_t warps = (int64_t)p->sm_count * piece_blocks_per_sm(p, max_per_sm) * p->warps_per_block;
-    const bool small = n_subgrids <= kPieceLists && n_vis <= warps * most;
-    const int64_t share = (n_vis + warps - 1) / warps;
+    const int64_t rounds = most == kPieceMost && n_subgrids <= kRoundLists ? kPieceRounds : 1;
+    const bool small = n_subgrids <= kPieceLists && n_vis <= warps * most * rounds;
+    const int64_t even = (n_vis + warps - 1) / warps, share = even < most ? even : most;
     return dg::Pieces{vis_offsets, n_subgrids, small ? (int)(share > least ? share : least) : 0, n_vis};
 }
 

@@ -153,6 +153,7 @@ struct PieceClaimerT {
     const Pieces &pieces;
     int lane;
     long long first, last;      // the piece
+    long long stride;           // to this warp's next one
     long long lo, hi;           // lane: its list's part of the piece (group of 32 lists before `next`)
     int next;                   // lists not yet looked at
     unsigned todo;              // lists of the group with visibilities left to batch
@@ -161,14 +162,20 @@ struct PieceClaimerT {
     {
         const long long k = (long long)(threadIdx.x / kWarp) * gridDim.x + blockIdx.x;
         first = k * p.per_warp;
+        stride = (long long)(blockDim.x / kWarp) * gridDim.x * p.per_warp;
         last = min(first + p.per_warp, (long long)p.n_vis);
     }
 
     __device__ Batch claim()
     {
         while (todo == 0) {
-            if (next >= pieces.n_subgrids || first >= last)
-                return Batch{0, 0, 0, 0};
+            if (next >= pieces.n_subgrids || first >= last) {
+                first += stride;
+                if (first >= pieces.n_vis)
+                    return Batch{0, 0, 0, 0};
+                last = min(first + pieces.per_warp, (long long)pieces.n_vis);
+                next = 0;
+            }
             const int s = next + lane;
             lo = hi = 0;
             if (s < pieces.n_subgrids) {

@@ -1187,6 +1187,8 @@ def test_steps_of_many_runs(dtype, comp, nz):
 @pytest.mark.parametrize("counts", [
     [1], [16], [17, 0, 0, 47], [63], [64], [65], [3] * 100, [0, 5] * 40 + [1000], [20000], [4000, 0, 3, 9000, 1],
     [7] * 256, [7] * 257,                                       # the most lists of a call by pieces, and one more
+    [200003], [90000, 0, 64, 99940, 7, 250001],                 # several pieces per warp
+    [13000] * 16, [13000] * 17,                                 # the most lists of those, and one more
 ])
 def test_small_calls_by_pieces(counts):
     # pieces that span several lists, empty lists, lists cut by pieces, more
@@ -1211,7 +1213,7 @@ def test_small_calls_by_pieces(counts):
         grid = p.grid(torch.from_numpy(y).to(d), uvw, offs, len(counts)).cpu().numpy()
         assert p.status() == n_bad
         # a larger call of the same lists, twice over, goes by the chunk table
-        reps = 1 + 200000 // w.n_vis
+        reps = 1 + 700000 // w.n_vis
         big = torch.from_numpy(np.tile(uvw_np, (reps, 1))).to(d)
         many = torch.from_numpy(np.concatenate([[0], np.full(len(counts) - 1, 0), [w.n_vis * reps]])).to(d)
         if len(counts) == 1:
