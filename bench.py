@@ -48,8 +48,8 @@ TRAFFIC_KERNEL_SOURCES = ("paper_2102_12739_gb300/csrc/degrid.cu",
                           "paper_2102_12739_gb300/csrc/footprint.cuh",
                           "paper_2102_12739_gb300/csrc/pipeline.cuh",
                           "paper_2102_12739_gb300/csrc/internal.cuh")
-TRAFFIC_SHA = "5f84fad245c2e04d"
-TRAFFIC_BYTES_PER_VIS = (98.423808e6 + 11.627776e6) / 4_000_000
+TRAFFIC_SHA = "7a9396e2311d4492"
+TRAFFIC_BYTES_PER_VIS = (98.419200e6 + 11.268096e6) / 4_000_000
 FP32_LANES_PER_SM = 128
 L2_FLUSH_BYTES = 256 << 20
 # (chunk, warps per CTA, CTAs per SM, direct-arm threshold) tried on the headline workload
